@@ -73,12 +73,12 @@ def draw(rng):
     def log(lo, hi):
         return math.exp(rng.uniform(math.log(lo), math.log(hi)))
 
-    # per kind: range of nx, multiple both sizes are of, largest right-hand-side count, largest nx nz nrhs
+    # per kind: range of nx, multiple that nz is of, largest right-hand-side count, largest nx nz nrhs
     lo, hi, div, most, points = {
         "apply": (64, 1360, 4, 256, 25e6), "residual": (64, 1360, 4, 256, 25e6), "vcycle": (64, 1360, 4, 256, 25e6),
         "samples": (64, 1024, 4, 64, 8e6), "solve": (64, 400, 4, 96, 3e6), "misfit": (64, 336, 4, 64, 2e6),
         "precond": (64, 1024, 8, 64, 16e6), "loss_grad": (64, 1024, 8, 32, 8e6)}[kind]
-    nx = max(lo, int(log(lo, hi)) // div * div)
+    nx = max(lo, int(log(lo, hi)) // 8 * 8)
     nz = max(32, int(nx * rng.uniform(0.4, 1.0)) // div * div)
     nrhs = max(1, int(log(1, most + 1)))
     nrhs = max(1, min(nrhs, most, int(points / (nx * nz))))
