@@ -230,6 +230,11 @@ int coarsest_solve(helm_ctx* c, int l, float2* u_out, const float2* f, int nb, c
     Level& L = c->lev[l];
     size_t Nc = (size_t)L.nx * L.nz;
     if (c->opt.coarse_kind == HELM_COARSE_GMRES) {
+        // one cluster per RHS where the grid fits one (an odd number of nodes stays refused below)
+        if (Nc % 2 == 0) {
+            const int st = launch_coarse_cluster(c, l, f, u_out, nb, mask);
+            if (st != HELM_EUNSUPPORTED) return st;
+        }
         // f is stored in Vc[0]; plain GMRES(k) from zero, one thread block per RHS
         if (f != c->Vc) HELM_TRY(launch_copy_masked(c, c->Vc, f, Nc, nb, mask));
         return launch_coarse_gmres(c, l, u_out, nb, mask);

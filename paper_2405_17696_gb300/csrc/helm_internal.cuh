@@ -369,6 +369,7 @@ int launch_arnoldi_update_ex(const helm_ctx* c, KState& st, const float2* w, flo
                              int nx, int nz, int nb, const int* iters_base, int max_iter, int* status);
 int launch_lsq(const helm_ctx* c, KState& st, int nb);
 int launch_normalize_v0(const helm_ctx* c, KState& st, float2* v0, size_t n, int nb);
+int launch_coarse_cluster(const helm_ctx* c, int level, const float2* f, float2* u_out, int nb, const int* mask);
 int launch_coarse_gmres(const helm_ctx* c, int level, float2* u_out, int nb, const int* mask);
 int launch_combine(const helm_ctx* c, const KState& st, float2* out, const float2* Zb, size_t zstride,
                    size_t n, int nb, const int* mask);
