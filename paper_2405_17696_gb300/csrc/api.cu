@@ -268,6 +268,13 @@ int smooth_and_recurse(helm_ctx* c, const Op& op, int l, float2* u_out, const fl
     Level& L = c->lev[l];
     Level& C = c->lev[l + 1];
     const int pre = c->opt.pre, post = c->opt.post, n = pre + post;
+    if (pre == 2 && post == 2 && !u0 && !stencil_tuning_on()) {
+        // the default cycle: one pass per leg (other sweep counts and initial guesses take the kernels below,
+        // whose block shapes helm_autotune times)
+        HELM_TRY(launch_leg_down(c, op, f, L.t, C.f, nb, mask));
+        HELM_TRY(vcycle_level(c, l + 1, C.u, nullptr, C.f, nb, mask));
+        return launch_leg_up(c, op, f, L.t, C.u, u_out, nb, mask);
+    }
     float2* bufs[2] = {u_out, L.t};
     const float2* cur = u0;
     int done = 0;

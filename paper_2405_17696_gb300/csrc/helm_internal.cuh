@@ -354,6 +354,13 @@ int launch_jacobi(const helm_ctx* c, const Op& op, float2* u_out, const float2* 
 template <class Op>
 int launch_restrict_residual(const helm_ctx* c, const Op& op, float2* rc, const float2* u, const float2* f,
                              int nx, int nz, int nb, const int* mask);
+// A level's two legs with two sweeps each, one pass per leg (k_legs.cu): down u2 = two sweeps from zero,
+// rc = R (f - A u2); up u = two sweeps from u2 + P ec (u2 and u distinct).  nx and nz even.
+template <class Op>
+int launch_leg_down(const helm_ctx* c, const Op& op, const float2* f, float2* u2, float2* rc, int nb, const int* mask);
+template <class Op>
+int launch_leg_up(const helm_ctx* c, const Op& op, const float2* f, const float2* u2, const float2* ec, float2* u, int nb,
+                  const int* mask);
 int launch_prolong_add(const helm_ctx* c, float2* u, const float2* ec, int nx, int nz, int nb, const int* mask);
 int launch_copy_masked(const helm_ctx* c, float2* dst, const float2* src, size_t n_per_rhs, int nb, const int* mask);
 
@@ -388,6 +395,7 @@ void cnn_retrain_free(helm_ctx* c);         // cnn_retrain.cu
 // Block-shape autotuning of the Jacobi sweeps (k_multigrid.cu): while on, the first launch
 // on a grid times the candidate shapes and records the fastest (process-wide table).
 void stencil_tuning(bool on);
+bool stencil_tuning_on();
 int stencil_tuned_count();
 void stencil_tune_reset();
 

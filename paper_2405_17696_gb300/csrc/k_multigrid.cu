@@ -373,6 +373,7 @@ int tune_shape(const helm_ctx* c, int kernel, int nx, int nz, F launch) {
 }  // namespace
 
 void stencil_tuning(bool on) { g_stencil_tuning.store(on ? 1 : 0); }
+bool stencil_tuning_on() { return g_stencil_tuning.load() != 0; }
 int stencil_tuned_count() {
     std::lock_guard<std::mutex> lk(g_shape_mu);
     return (int)g_shape.size();
