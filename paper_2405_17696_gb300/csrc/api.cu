@@ -1,6 +1,7 @@
 // C ABI of libhelm: context set-up (medium, frequencies, Galerkin multigrid
 // hierarchy, workspace), the batched FGMRES driver, the V-cycle driver and
 // the operator application.  See include/helm.h for the contract.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -192,7 +193,7 @@ int alloc_kstate(helm_ctx* c, KState& st, int k, int max_tiles) {
     HELM_TRY(dalloc(c, &st.steps, cap));
     HELM_TRY(dalloc(c, &st.tol_abs, cap));
     HELM_TRY(dalloc(c, &st.inv_est, cap));
-    HELM_TRY(dalloc(c, &st.partials, cap * (size_t)max_tiles * (KMAX + 2)));
+    HELM_TRY(dalloc(c, &st.partials, std::max<size_t>(cap * (size_t)max_tiles, ARNOLDI_SMALL_TILES) * (KMAX + 2)));
     HELM_TRY(dalloc(c, &st.counters, cap));
     HELM_CK(cudaMemsetAsync(st.counters, 0, cap * sizeof(unsigned), c->stream));
     HELM_CK(cudaMemsetAsync(st.active, 0, cap * sizeof(int), c->stream));
@@ -614,7 +615,7 @@ int helm_setup(helm_ctx** out, const float* kappa, const float* gamma, int nx, i
         os.max_tiles = tiles_of(nx, nz);
         if ((st = dalloc(c, &os.bnorm2, cap)) || (st = dalloc(c, &os.rnorm2, cap)) ||
             (st = dalloc(c, &os.iters, cap)) || (st = dalloc(c, &os.status, cap)) ||
-            (st = dalloc(c, &os.outer_active, cap)) || (st = dalloc(c, &os.partials, cap * os.max_tiles)) ||
+            (st = dalloc(c, &os.outer_active, cap)) || (st = dalloc(c, &os.partials, (cap + 1) * std::max<size_t>(os.max_tiles, ARNOLDI_SMALL_TILES))) ||
             (st = dalloc(c, &os.counters, cap)) || (st = dalloc(c, &os.rprev, cap)) ||
             (st = dalloc(c, &os.guard, cap)))
             return fail(st);

@@ -17,6 +17,7 @@ constexpr int KMAX = 16;          // largest restart / coarse-GMRES length suppo
 constexpr int TILE_X = 32;        // threads per block along x
 constexpr int TILE_Y = 8;         // threads per block along z
 constexpr int ROWS = 8;           // rows of z handled per thread in tiled kernels
+constexpr int ARNOLDI_SMALL_TILES = 152;   // tiles of a batch whose Arnoldi kernels take fewer rows per thread, at most
 
 void set_error(const std::string& msg);
 
@@ -191,7 +192,7 @@ struct KState {
     int* steps;            // [cap] steps taken in this cycle
     double* tol_abs;       // [cap] stop when |g_{j+1}| <= tol_abs
     double* inv_est;       // [cap] 1 / (estimate of ||w'||) applied when v~_{j+1} is written
-    double2* partials;     // [cap][max_tiles][KMAX + 2]
+    double2* partials;     // [RHS][tiles of the launch][KMAX + 2]
     unsigned* counters;    // [cap] arrival counters of the last-block reductions
     int max_tiles;
 };
@@ -205,7 +206,7 @@ struct OuterState {
     int* outer_active;     // 1 while not finished
     double* rprev;         // ||b - A x|| at the previous restart (0 before the first)
     int* guard;            // 1 once a restart cycle barely lowered the residual (network composition guarded)
-    double2* partials;     // [cap][max_tiles][2]
+    double2* partials;     // [RHS][tiles of the launch]
     unsigned* counters;
     int max_tiles;
 };
@@ -365,6 +366,7 @@ int launch_prolong_add(const helm_ctx* c, float2* u, const float2* ec, int nx, i
 int launch_copy_masked(const helm_ctx* c, float2* dst, const float2* src, size_t n_per_rhs, int nb, const int* mask);
 
 // Krylov pieces
+int arnoldi_rows(int xtiles, int nz, int nb);   // rows per thread of the tiled kernels (k_krylov.cu)
 int launch_kstate_init(const helm_ctx* c, KState& st, const float2* v0, int nx, int nz, int nb,
                        const int* mask);
 template <class Op>

@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "helm_internal.cuh"
+#include "reduce.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -39,40 +40,6 @@ namespace {
 constexpr int CC_MAX = 16;          // CTAs per cluster at most (the non-portable limit)
 constexpr int CC_WARPS = 24;        // warps per CTA at most
 constexpr size_t CC_SMEM = 200 * 1024;   // dynamic shared memory at most
-
-// Two-term numbers (h + l, |l| <= ulp(h) / 2; about 46 bits): FP64 instructions take some 64 cycles each
-// on this GPU and the serial parts of the solve would wait on them.
-struct ff {
-    float h, l;
-};
-__device__ __forceinline__ ff ff_quick(float h, float l) {
-    ff r;
-    r.h = h + l;
-    r.l = l - (r.h - h);
-    return r;
-}
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-    const float s = a.h + b.h, bb = s - a.h;
-    return ff_quick(s, (a.h - (s - bb)) + (b.h - bb) + (a.l + b.l));
-}
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-    const float p = a.h * b.h;
-    return ff_quick(p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p))));
-}
-__device__ __forceinline__ ff ff_rcp(ff a) {
-    const float y = 1.0f / a.h;
-    return ff_quick(y, y * (fmaf(-y, a.h, 1.0f) - y * a.l));
-}
-// 1 / sqrt(a), a > 0: one Newton step on the FP32 value
-__device__ __forceinline__ ff ff_rsqrt(ff a) {
-    const float y = rsqrtf(a.h);
-    const ff t = ff_mul(a, ff_mul({y, 0.f}, {y, 0.f}));
-    return ff_quick(y, 0.5f * y * ((1.0f - t.h) - t.l));
-}
-__device__ __forceinline__ ff ff_shfl(ff a, int src) {
-    return {__shfl_sync(0xffffffffu, a.h, src), __shfl_sync(0xffffffffu, a.l, src)};
-}
 
 struct CoarsePlan {
     int npt = 0;        // rows of a thread's strip (0: the layer is not taken)

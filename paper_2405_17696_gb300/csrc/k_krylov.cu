@@ -29,52 +29,117 @@ __device__ __forceinline__ double2* kcol(const KState& st, int b, int j) {
     return st.H + ((size_t)b * st.k + j) * (st.k + 1);
 }
 
-// One Givens step on column j of RHS b after h_{j+1,j} is known (Saad 2003,
-// Sec. 6.5.3, complex form: rotation [c s; -conj(s) c] with real c).
-__device__ void givens_step(const KState& st, int b, int j, double hnext, double s_next, const int* iters_base,
-                            int max_iter, int* status) {
-    double2* hc = kcol(st, b, j);
-    hc[j + 1] = make_double2(hnext, 0.0);
+// One Givens step on column J of RHS b once n2 = ||v~_{J+1}||^2 is known (Saad 2003,
+// Sec. 6.5.3, complex form: rotation [c s; -conj(s) c] with real c).  All threads
+// of the block call it: they fetch the column and the rotations at once, thread 0
+// computes (a chain of FP64 operations of some 64 cycles each; reciprocal square
+// roots instead of quotients and roots of 400).
+template <int J>
+__device__ void givens_step(const KState& st, int b, double n2, double inv_est, const int* iters_base, int max_iter,
+                            int* status) {
+    __shared__ double2 hc_s[J + 1], sn_s[J + 1];
+    __shared__ double cs_s[J + 1];
+    const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+    double2* hc = kcol(st, b, J);
     double* cs = st.cs + (size_t)b * st.k;
     double2* sn = st.sn + (size_t)b * st.k;
-    for (int i = 0; i < j; ++i) {
-        double2 a = hc[i], bb = hc[i + 1];
-        double c = cs[i];
-        double2 s = sn[i];
-        hc[i] = dadd(make_double2(c * a.x, c * a.y), dmul(s, bb));
-        hc[i + 1] = dadd(make_double2(-(s.x * a.x + s.y * a.y), -(s.x * a.y - s.y * a.x)),
-                         make_double2(c * bb.x, c * bb.y));
+    if (tid <= J) {
+        hc_s[tid] = hc[tid];
+        if (tid < J) {
+            cs_s[tid] = cs[tid];
+            sn_s[tid] = sn[tid];
+        }
     }
-    double2 a = hc[j];
-    double hb = hc[j + 1].x;
-    double na = sqrt(dabs2(a));
-    double nu = sqrt(na * na + hb * hb);
+    double2* g = st.g + (size_t)b * (st.k + 1);
+    double2 gj = make_double2(0.0, 0.0);
+    double tol = 0.0;
+    int taken = 0;
+    if (tid == 0) {
+        gj = g[J];
+        tol = st.tol_abs[b];
+        taken = iters_base ? iters_base[b] : 0;
+    }
+    __syncthreads();
+    if (tid != 0) return;
+    double2 a = hc_s[0];
+#pragma unroll 1
+    for (int i = 0; i < J; ++i) {
+        const double2 bb = hc_s[i + 1];
+        const double c = cs_s[i];
+        const double2 s = sn_s[i];
+        hc[i] = dadd(make_double2(c * a.x, c * a.y), dmul(s, bb));
+        a = dadd(make_double2(-(s.x * a.x + s.y * a.y), -(s.x * a.y - s.y * a.x)), make_double2(c * bb.x, c * bb.y));
+    }
+    const double rn = n2 > 0.0 ? rsqrt(n2) : 0.0, nrm = n2 * rn;   // ||v~_{J+1}||
+    const double hb = nrm / inv_est;                               // ||w'|| = est ||v~_{J+1}||
+    const double na2 = dabs2(a), nu2 = na2 + hb * hb;
+    const double rnu = nu2 > 0.0 ? rsqrt(nu2) : 0.0, nu = nu2 * rnu;
     double c;
     double2 s;
-    if (na == 0.0) {
+    if (na2 == 0.0) {
         c = 0.0;
         s = make_double2(1.0, 0.0);
-        hc[j] = make_double2(hb, 0.0);
+        hc[J] = make_double2(hb, 0.0);
     } else {
-        c = na / nu;
-        s = make_double2(a.x / na * hb / nu, a.y / na * hb / nu);
-        hc[j] = make_double2(a.x / na * nu, a.y / na * nu);
+        const double rna = rsqrt(na2);
+        const double2 ph = make_double2(a.x * rna, a.y * rna);   // a / |a|
+        c = na2 * rna * rnu;
+        s = make_double2(ph.x * (hb * rnu), ph.y * (hb * rnu));
+        hc[J] = make_double2(ph.x * nu, ph.y * nu);
     }
-    hc[j + 1] = make_double2(0.0, 0.0);
-    cs[j] = c;
-    sn[j] = s;
-    double2* g = st.g + (size_t)b * (st.k + 1);
-    double2 gj = g[j];
-    g[j + 1] = make_double2(-(s.x * gj.x + s.y * gj.y), -(s.x * gj.y - s.y * gj.x));  // -conj(s) g_j
-    g[j] = make_double2(c * gj.x, c * gj.y);
-    double est = sqrt(dabs2(g[j + 1]));
-    st.steps[b] = j + 1;
-    st.s[(size_t)b * (st.k + 1) + j + 1] = s_next;
+    hc[J + 1] = make_double2(0.0, 0.0);
+    cs[J] = c;
+    sn[J] = s;
+    const double2 gn = make_double2(-(s.x * gj.x + s.y * gj.y), -(s.x * gj.y - s.y * gj.x));  // -conj(s) g_j
+    g[J + 1] = gn;
+    g[J] = make_double2(c * gj.x, c * gj.y);
+    const double est = sqrt(dabs2(gn));
+    st.steps[b] = J + 1;
+    st.s[(size_t)b * (st.k + 1) + J + 1] = nrm > 0.0 ? rn : 0.0;
     bool finite = isfinite(est) && isfinite(hb) && isfinite(nu);
     bool tiny = !(hb > 1e-300);
-    bool cap = iters_base && (iters_base[b] + j + 1 >= max_iter);
+    bool cap = iters_base && (taken + J + 1 >= max_iter);
     if (!finite && status) status[b] = HELM_EBREAKDOWN;
-    if (!finite || tiny || est <= st.tol_abs[b] || cap || j + 1 >= st.k) st.active[b] = 0;
+    if (!finite || tiny || est <= tol || cap || J + 1 >= st.k) st.active[b] = 0;
+}
+
+// (With FP64 shuffles the J + 2 sums of a block took some 7 us; at J = 9, 512 x 256 and 192 right-hand
+// sides on one GB300 the pass took 463 us with them and takes 310, 302 MB per basis vector at 7.8 TB/s
+// counting what L2 keeps; 20 us and 10 for one right-hand side of 160 x 160, with one row per thread.)
+// The block's part of the inner products acc[i] = <v~_i, w>, i <= J, acc[J + 1] = ||w||^2; the last block of
+// the RHS scales them to column J of the Hessenberg matrix and estimates ||w'||.
+template <int J>
+__device__ __forceinline__ void dots_finish(const KState& st, int b, const float2 (&acc)[J + 2]) {
+    __shared__ double2 sm[NWARPS * ((J + 5) / 4 * 4)];
+    __shared__ double2 hs[J + 2];
+    __shared__ double hsq[J + 2];
+    const int ntiles = gridDim.x * gridDim.y;
+    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
+    double2* part = st.partials + (size_t)b * ntiles * (KMAX + 2);
+    if (!reduce_block_last_f32<J + 2>(acc, part + (size_t)tile * (KMAX + 2), st.counters + b, ntiles, sm)) return;
+    sum_tiles(part, ntiles, KMAX + 2, J + 2, hs);
+    const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+    if (tid <= J + 1) {
+        double2 h = hs[tid];
+        if (tid <= J) {
+            const double sc = st.s[(size_t)b * (st.k + 1) + tid];
+            h = make_double2(h.x * sc, h.y * sc);
+            kcol(st, b, J)[tid] = h;
+            hsq[tid] = dabs2(h);
+        } else {
+            hsq[tid] = h.x;   // ||w||^2
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double w2 = hsq[J + 1], proj = 0.0;
+        for (int i = 0; i <= J; ++i) proj += hsq[i];
+        double est2 = w2 - proj;
+        // a cancelled estimate only changes the scale the vector is stored at
+        if (!(est2 > 1e-12 * w2)) est2 = 1e-12 * w2;
+        const double est = sqrt(est2);
+        st.inv_est[b] = (est > 0.0 && isfinite(est)) ? 1.0 / est : 1.0;
+    }
 }
 
 // w = A z for RHS b and the inner products h_{i,j} = s_i <v~_i, w>, i <= j,
@@ -85,7 +150,7 @@ template <class Op, int J>
 __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_dots_kernel(Op op, KState st, const float2* __restrict__ z,
                                                                    float2* __restrict__ w,
                                                                    const float2* __restrict__ V, size_t vstride,
-                                                                   int nx, int nz, Tally tl) {
+                                                                   int nx, int nz, int rows, Tally tl) {
     const int b = blockIdx.z;
     if (!st.active[b]) return;
     tally_once(tl, blockIdx.x == 0 && blockIdx.y == 0);
@@ -94,13 +159,13 @@ __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_dots_kernel(Op op, KState
     float2* wb = w + (size_t)b * N;
     const float2* Vb = V + (size_t)b * N;
     const int ix = blockIdx.x * TILE_X + threadIdx.x;
-    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * ROWS;
+    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * rows;
     float2 acc[J + 2];   // acc[i] = <v~_i, w> for i <= J, acc[J+1] = ||w||^2
 #pragma unroll
     for (int i = 0; i < J + 2; ++i) acc[i] = make_float2(0.f, 0.f);
     if (ix < nx) {
 #pragma unroll 2
-        for (int r = 0; r < ROWS; ++r) {
+        for (int r = 0; r < rows; ++r) {
             int iz = iz0 + r;
             if (iz >= nz) break;
             size_t p = (size_t)iz * nx + ix;
@@ -117,43 +182,14 @@ __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_dots_kernel(Op op, KState
             acc[J + 1].x += y.x * y.x + y.y * y.y;
         }
     }
-    __shared__ double2 sm[NWARPS * (J + 2)];
-    __shared__ double hsq[J + 2];
-    const int ntiles = gridDim.x * gridDim.y;
-    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
-    double2* part = st.partials + ((size_t)b * st.max_tiles) * (KMAX + 2);
-    bool last = reduce_block_last<J + 2>(acc, J + 2, part + (size_t)tile * (KMAX + 2), st.counters + b, ntiles, sm);
-    if (last) {
-        const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-        if (tid <= J + 1) {
-            double2 h = sum_partials(part, ntiles, KMAX + 2, tid);
-            if (tid <= J) {
-                double sc = st.s[(size_t)b * (st.k + 1) + tid];
-                h = make_double2(h.x * sc, h.y * sc);
-                kcol(st, b, J)[tid] = h;
-                hsq[tid] = dabs2(h);
-            } else {
-                hsq[tid] = h.x;   // ||w||^2
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double w2 = hsq[J + 1], proj = 0.0;
-            for (int i = 0; i <= J; ++i) proj += hsq[i];
-            double est2 = w2 - proj;
-            // a cancelled estimate only changes the scale the vector is stored at
-            if (!(est2 > 1e-12 * w2)) est2 = 1e-12 * w2;
-            double est = sqrt(est2);
-            st.inv_est[b] = (est > 0.0 && isfinite(est)) ? 1.0 / est : 1.0;
-        }
-    }
+    dots_finish<J>(st, b, acc);
 }
 
 // v~_{j+1} = (w - sum_i h_{i,j} s_i v~_i) / est, its norm, then the Givens step.
 template <int J>
-__global__ void __launch_bounds__(NTHREADS, 3) arnoldi_update_kernel(KState st, const float2* __restrict__ w,
+__global__ void __launch_bounds__(NTHREADS, J <= 5 ? 4 : 3) arnoldi_update_kernel(KState st, const float2* __restrict__ w,
                                                                      float2* __restrict__ V, size_t vstride,
-                                                                     int nx, int nz, const int* iters_base,
+                                                                     int nx, int nz, int rows, const int* iters_base,
                                                                      int max_iter, int* status, Tally tl) {
     const int b = blockIdx.z;
     if (!st.active[b]) return;
@@ -173,11 +209,11 @@ __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_update_kernel(KState st, 
     float2* Vb = V + (size_t)b * N;
     float2* vout = Vb + (size_t)(J + 1) * vstride;
     const int ix = blockIdx.x * TILE_X + threadIdx.x;
-    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * ROWS;
+    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * rows;
     float acc = 0.f;
     if (ix < nx) {
 #pragma unroll 2
-        for (int r = 0; r < ROWS; ++r) {
+        for (int r = 0; r < rows; ++r) {
             int iz = iz0 + r;
             if (iz >= nz) break;
             size_t p = (size_t)iz * nx + ix;
@@ -197,17 +233,15 @@ __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_update_kernel(KState st, 
             acc += y.x * y.x + y.y * y.y;
         }
     }
-    __shared__ double2 sm[NWARPS];
-    double2 vals[1] = {make_double2((double)acc, 0.0)};
+    __shared__ double2 sm[NWARPS * 4];
+    __shared__ double2 n2;
+    const float2 vals[1] = {make_float2(acc, 0.f)};
     const int ntiles = gridDim.x * gridDim.y;
     const int tile = blockIdx.y * gridDim.x + blockIdx.x;
-    double2* part = st.partials + ((size_t)b * st.max_tiles) * (KMAX + 2);
-    bool last = reduce_block_last<1>(vals, 1, part + (size_t)tile * (KMAX + 2), st.counters + b, ntiles, sm);
-    if (last && tid == 0) {
-        double nrm = sqrt(sum_partials(part, ntiles, KMAX + 2, 0).x);   // ||v~_{j+1}||
-        double hnext = nrm / inv;                                       // ||w'|| = est ||v~_{j+1}||
-        givens_step(st, b, J, hnext, nrm > 0.0 ? 1.0 / nrm : 0.0, iters_base, max_iter, status);
-    }
+    double2* part = st.partials + (size_t)b * ntiles * (KMAX + 2);
+    if (!reduce_block_last_f32<1>(vals, part + (size_t)tile * (KMAX + 2), st.counters + b, ntiles, sm)) return;
+    sum_tiles(part, ntiles, KMAX + 2, 1, &n2);
+    givens_step<J>(st, b, n2.x, inv, iters_base, max_iter, status);
 }
 
 // ||v0||^2 per RHS, then g_0 = ||v0||, s_0 = 1/||v0||, steps = 0, active = mask && ||v0|| > 0.
@@ -266,20 +300,32 @@ __global__ void normalize_v0_kernel(KState st, float2* __restrict__ v0, size_t n
     if (blockIdx.x == 0 && threadIdx.x == 0) st.s[(size_t)b * (st.k + 1)] = 1.0;
 }
 
-// Back substitution R y = g for every RHS (FP64, one thread per RHS).
+// Back substitution R y = g (FP64), one warp per RHS: lane i carries row i, and the
+// reciprocals of the diagonal are taken by all lanes at once.
 __global__ void lsq_kernel(KState st, int nb) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (b >= nb) return;
-    int n = st.steps[b];
+    const int n = st.steps[b];
+    if (n == 0) return;
     double2* y = st.y + (size_t)b * st.k;
-    const double2* g = st.g + (size_t)b * (st.k + 1);
-    for (int i = n - 1; i >= 0; --i) {
-        double2 acc = g[i];
-        for (int c = i + 1; c < n; ++c) acc = dsub(acc, dmul(kcol(st, b, c)[i], y[c]));
-        double2 d = kcol(st, b, i)[i];
-        double dd = dabs2(d);
-        y[i] = dd > 0.0 ? make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd)
-                        : make_double2(0.0, 0.0);
+    double2 acc = make_double2(0.0, 0.0), r = make_double2(0.0, 0.0);
+    if (lane < n) {
+        acc = st.g[(size_t)b * (st.k + 1) + lane];
+        const double2 d = kcol(st, b, lane)[lane];
+        const double dd = dabs2(d), i = dd > 0.0 ? 1.0 / dd : 0.0;
+        r = make_double2(d.x * i, -d.y * i);                     // 1 / d
+    }
+    double2 hcol[KMAX];                                          // row `lane` of R
+#pragma unroll
+    for (int c = 0; c < KMAX; ++c)
+        hcol[c] = c < n && lane < c ? kcol(st, b, c)[lane] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int c = KMAX - 1; c >= 0; --c) {
+        if (c >= n) continue;
+        const double2 yc = dmul(acc, r);
+        const double2 v = make_double2(__shfl_sync(0xffffffffu, yc.x, c), __shfl_sync(0xffffffffu, yc.y, c));
+        acc = lane == c ? acc : dsub(acc, dmul(hcol[c], v));
+        if (lane == c) y[c] = v;
     }
 }
 
@@ -349,7 +395,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_dots_fine2_kernel(OpFine5
                                                                         const float2* __restrict__ z,
                                                                         float2* __restrict__ w,
                                                                         const float2* __restrict__ V,
-                                                                        size_t vstride, int nx, int nz, Tally tl) {
+                                                                        size_t vstride, int nx, int nz, int rows, Tally tl) {
     const int b = blockIdx.z;
     if (!st.active[b]) return;
     tally_once(tl, blockIdx.x == 0 && blockIdx.y == 0);
@@ -358,13 +404,13 @@ __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_dots_fine2_kernel(OpFine5
     float2* wb = w + (size_t)b * N;
     const float2* Vb = V + (size_t)b * N;
     const int ix = 2 * (blockIdx.x * TILE_X + threadIdx.x);
-    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * ROWS;
+    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * rows;
     float2 acc[J + 2];
 #pragma unroll
     for (int i = 0; i < J + 2; ++i) acc[i] = make_float2(0.f, 0.f);
     if (ix < nx) {
 #pragma unroll 2
-        for (int r = 0; r < ROWS; ++r) {
+        for (int r = 0; r < rows; ++r) {
             const int iz = iz0 + r;
             if (iz >= nz) break;
             const size_t p = (size_t)iz * nx + ix;
@@ -382,39 +428,20 @@ __global__ void __launch_bounds__(NTHREADS, 3) arnoldi_dots_fine2_kernel(OpFine5
             acc[J + 1].x += y0.x * y0.x + y0.y * y0.y + y1.x * y1.x + y1.y * y1.y;
         }
     }
-    __shared__ double2 sm[NWARPS * (J + 2)];
-    __shared__ double hsq[J + 2];
-    const int ntiles = gridDim.x * gridDim.y;
-    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
-    double2* part = st.partials + ((size_t)b * st.max_tiles) * (KMAX + 2);
-    bool last = reduce_block_last<J + 2>(acc, J + 2, part + (size_t)tile * (KMAX + 2), st.counters + b, ntiles, sm);
-    if (last) {
-        const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-        if (tid <= J + 1) {
-            double2 h = sum_partials(part, ntiles, KMAX + 2, tid);
-            if (tid <= J) {
-                double sc = st.s[(size_t)b * (st.k + 1) + tid];
-                h = make_double2(h.x * sc, h.y * sc);
-                kcol(st, b, J)[tid] = h;
-                hsq[tid] = dabs2(h);
-            } else {
-                hsq[tid] = h.x;
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double w2 = hsq[J + 1], proj = 0.0;
-            for (int i = 0; i <= J; ++i) proj += hsq[i];
-            double est2 = w2 - proj;
-            if (!(est2 > 1e-12 * w2)) est2 = 1e-12 * w2;
-            double est = sqrt(est2);
-            st.inv_est[b] = (est > 0.0 && isfinite(est)) ? 1.0 / est : 1.0;
-        }
-    }
+    dots_finish<J>(st, b, acc);
 }
 
 static dim3 tiled_grid(int nx, int nz, int nb) {
     return dim3((nx + TILE_X - 1) / TILE_X, (nz + TILE_Y * ROWS - 1) / (TILE_Y * ROWS), nb);
+}
+
+// Rows per thread of the Arnoldi kernels: 8, fewer while the batch has less than a block for every other SM (a small
+// grid waits for the loads of one thread's rows).  Fewer than 8 rows means at most ARNOLDI_SMALL_TILES tiles.
+int arnoldi_rows(int xtiles, int nz, int nb) {
+    for (int rows = ROWS; rows > 1; rows /= 2)
+        if ((long long)xtiles * ((nz + TILE_Y * rows - 1) / (TILE_Y * rows)) * nb >= ARNOLDI_SMALL_TILES / 2)
+            return rows;
+    return 1;
 }
 
 #define HELM_J_CASES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15)
@@ -428,12 +455,13 @@ int launch_arnoldi_dots(const helm_ctx* c, const Op& op, KState& st, const float
                            8ull * nx * nz * (j + 3));
     if constexpr (std::is_same<Op, OpFine5>::value) {
         if (nx % 2 == 0) {
-            const dim3 grid2((nx / 2 + TILE_X - 1) / TILE_X, (nz + TILE_Y * ROWS - 1) / (TILE_Y * ROWS), nb),
+            const int rows = arnoldi_rows((nx / 2 + TILE_X - 1) / TILE_X, nz, nb);
+            const dim3 grid2((nx / 2 + TILE_X - 1) / TILE_X, (nz + TILE_Y * rows - 1) / (TILE_Y * rows), nb),
                 block2(TILE_X, TILE_Y);
             switch (j) {
 #define HELM_DOTS2_CASE(J)                                                                                  \
     case J:                                                                                                 \
-        { arnoldi_dots_fine2_kernel<J><<<grid2, block2, 0, c->stream>>>(op, st, z, w, V, vstride, nx, nz, tl); count_launch(); } \
+        { arnoldi_dots_fine2_kernel<J><<<grid2, block2, 0, c->stream>>>(op, st, z, w, V, vstride, nx, nz, rows, tl); count_launch(); } \
         break;
                 HELM_J_CASES(HELM_DOTS2_CASE)
 #undef HELM_DOTS2_CASE
@@ -445,11 +473,12 @@ int launch_arnoldi_dots(const helm_ctx* c, const Op& op, KState& st, const float
             return HELM_OK;
         }
     }
-    const dim3 grid = tiled_grid(nx, nz, nb), block(TILE_X, TILE_Y);
+    const int rows = arnoldi_rows((nx + TILE_X - 1) / TILE_X, nz, nb);
+    const dim3 grid((nx + TILE_X - 1) / TILE_X, (nz + TILE_Y * rows - 1) / (TILE_Y * rows), nb), block(TILE_X, TILE_Y);
     switch (j) {
 #define HELM_DOTS_CASE(J)                                                                                     \
     case J:                                                                                                   \
-        { arnoldi_dots_kernel<Op, J><<<grid, block, 0, c->stream>>>(op, st, z, w, V, vstride, nx, nz, tl); count_launch(); }   \
+        { arnoldi_dots_kernel<Op, J><<<grid, block, 0, c->stream>>>(op, st, z, w, V, vstride, nx, nz, rows, tl); count_launch(); }   \
         break;
         HELM_J_CASES(HELM_DOTS_CASE)
 #undef HELM_DOTS_CASE
@@ -470,11 +499,12 @@ int launch_arnoldi_update_ex(const helm_ctx* c, KState& st, const float2* w, flo
     const int kid = st.H == c->fine.H ? K_UPDATE_FINE : K_UPDATE_COARSE;
     LaunchScope scope(c, kid);
     const Tally tl = tally(c, kid, 8ull * nx * nz * (j + 3));
-    const dim3 grid = tiled_grid(nx, nz, nb), block(TILE_X, TILE_Y);
+    const int rows = arnoldi_rows((nx + TILE_X - 1) / TILE_X, nz, nb);
+    const dim3 grid((nx + TILE_X - 1) / TILE_X, (nz + TILE_Y * rows - 1) / (TILE_Y * rows), nb), block(TILE_X, TILE_Y);
     switch (j) {
 #define HELM_UPD_CASE(J)                                                                                        \
     case J:                                                                                                     \
-        { arnoldi_update_kernel<J><<<grid, block, 0, c->stream>>>(st, w, V, vstride, nx, nz, iters_base, max_iter, \
+        { arnoldi_update_kernel<J><<<grid, block, 0, c->stream>>>(st, w, V, vstride, nx, nz, rows, iters_base, max_iter, \
                                                                  status, tl); count_launch(); }                                  \
         break;
         HELM_J_CASES(HELM_UPD_CASE)
@@ -512,7 +542,7 @@ int launch_normalize_v0(const helm_ctx* c, KState& st, float2* v0, size_t n, int
 
 int launch_lsq(const helm_ctx* c, KState& st, int nb) {
     LaunchScope scope(c, K_LSQ);
-    { lsq_kernel<<<(nb + 127) / 128, 128, 0, c->stream>>>(st, nb); count_launch(); }
+    { lsq_kernel<<<(nb + 3) / 4, 128, 0, c->stream>>>(st, nb); count_launch(); }
     HELM_CK(cudaGetLastError());
     return HELM_OK;
 }
