@@ -25,61 +25,176 @@ __global__ void apply_fine_kernel(OpFine5 op, const float2* __restrict__ x, floa
     y[(size_t)b * N + (size_t)iz * op.nx + ix] = op.apply(x + (size_t)b * N, b, ix, iz);
 }
 
+// y = A x on node pairs (nx even): a thread carries three rows of its pair down `rows` rows, so that a
+// field is read about once (the neighbours' columns come from L1) with 16-byte accesses.  The rounded
+// operations are those of OpFine5::apply in apply_fine_kernel, spelled out: the training pairs made
+// from H x do not depend on which kernel made it.  512 x 256, 192 fields, one GB300:
+// 115 -> 68 us (403 MB: 5.9 TB/s).
+__global__ void __launch_bounds__(NTHREADS) apply_fine2_kernel(OpFine5 op, const float2* __restrict__ x,
+                                                               float2* __restrict__ y, int rows, const int* mask,
+                                                               Tally tl) {
+    const int b = blockIdx.z;
+    if (!mask[b]) return;
+    tally_once(tl, blockIdx.x == 0 && blockIdx.y == 0);
+    const int nx = op.nx, nz = op.nz;
+    const int ix = 2 * (blockIdx.x * TILE_X + threadIdx.x);
+    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * rows;
+    if (ix >= nx || iz0 >= nz) return;
+    const size_t N = (size_t)nx * nz;
+    const float2* xb = x + (size_t)b * N + ix;
+    float2* yb = y + (size_t)b * N + ix;
+    const float w = __ldg(op.omega + __ldg(op.rhs_freq + b)), w2 = __fmul_rn(w, w);
+    const float ax = op.ax, az = op.az;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto row = [&](int iz) { return iz >= 0 && iz < nz ? __ldg(reinterpret_cast<const float4*>(xb + (size_t)iz * nx)) : zero; };
+    // ax (2 c - l - r) + az (2 c - n - s)
+    auto lap = [&](float c, float l, float r, float n, float s) {
+        return __fmaf_rn(ax, __fsub_rn(__fmaf_rn(2.f, c, -l), r), __fmul_rn(az, __fsub_rn(__fmaf_rn(2.f, c, -n), s)));
+    };
+    float4 n = row(iz0 - 1), c = row(iz0);
+#pragma unroll 4
+    for (int rr = 0; rr < rows; ++rr) {
+        const int iz = iz0 + rr;
+        if (iz >= nz) break;
+        const float4 s = row(iz + 1);
+        const float2 l = ix > 0 ? __ldg(xb + (size_t)iz * nx - 1) : make_float2(0.f, 0.f);
+        const float2 r = ix + 2 < nx ? __ldg(xb + (size_t)iz * nx + 2) : make_float2(0.f, 0.f);
+        const float4 m = __ldg(reinterpret_cast<const float4*>(op.mg + (size_t)iz * nx + ix));
+        const float s0 = __fmul_rn(w2, __fmul_rn(m.x, m.x)), s1 = __fmul_rn(w2, __fmul_rn(m.z, m.z));
+        const float g0 = op.sl ? __fadd_rn(op.beta, op.incg ? m.y : 0.0f) : m.y;
+        const float g1 = op.sl ? __fadd_rn(op.beta, op.incg ? m.w : 0.0f) : m.w;
+        const float k0 = __fmul_rn(-s0, g0), k1 = __fmul_rn(-s1, g1);
+        float4 o;
+        o.x = __fsub_rn(lap(c.x, l.x, c.z, n.x, s.x), __fmaf_rn(s0, c.x, -__fmul_rn(k0, c.y)));
+        o.y = __fsub_rn(lap(c.y, l.y, c.w, n.y, s.y), __fmaf_rn(s0, c.y, __fmul_rn(k0, c.x)));
+        o.z = __fsub_rn(lap(c.z, c.x, r.x, n.z, s.z), __fmaf_rn(s1, c.z, -__fmul_rn(k1, c.w)));
+        o.w = __fsub_rn(lap(c.w, c.y, r.y, n.w, s.w), __fmaf_rn(s1, c.w, __fmul_rn(k1, c.z)));
+        *reinterpret_cast<float4*>(yb + (size_t)iz * nx) = o;
+        n = c;
+        c = s;
+    }
+}
+
+// float <-> double by integer operations: conversions run at the FP64 pipe's two per SM and cycle, which
+// bounds the residual below.  Zeros, denormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+    if (e - 1u >= 254u) return (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+// round to nearest even
+__device__ __forceinline__ float narrow(double d) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+    const unsigned e = (unsigned)(u >> 52) & 0x7ffu;
+    if (e - 897u >= 253u) return (float)d;            // (the largest finite exponent too: it may round up to infinity)
+    const unsigned long long v = u + 0x0fffffffull + ((u >> 29) & 1ull);
+    return __uint_as_float(((unsigned)(u >> 32) & 0x80000000u) | ((unsigned)((v >> 29) & 0xffffffffull) - (896u << 23) & 0x7fffffffu));
+}
+
 // r = b - H x evaluated in FP64 from the complex128 iterate x (b conjugated
 // when solving the adjoint system); r is stored in complex64 as the first
 // (unscaled) Krylov vector.  ||r||^2 and, on the first call, ||b||^2 are
 // reduced per RHS in FP64.
+//
+// Bound by the FP64 pipe (two operations per SM and cycle on this GPU): 17 per node and RHS as
+//   r = b + ax (xw + xe) + az (xn + xs) - (2 ax + 2 az - w^2 m) xc - i (w^2 m gamma) xc
+// with w^2 m and its products shared by a thread's two right-hand sides of one frequency, against
+// 34 in the order the operator is written, its conversions included.  512 x 256, 192 right-hand
+// sides, one GB300: 1.92 -> 1.31 ms a call, 1.47 -> 0.90 ms inside a solve.
+template <bool FIRST>
 __global__ void __launch_bounds__(NTHREADS) residual64_kernel(OpFine5 op, const double2* __restrict__ x,
                                                               const float2* __restrict__ bvec,
-                                                              float2* __restrict__ r, int conj_b, int first,
+                                                              float2* __restrict__ r, int conj_b, int nb, int rows,
                                                               double ax, double az, OuterState os, Tally tl) {
-    const int b = blockIdx.z;
-    if (!os.outer_active[b]) return;
-    tally_once(tl, blockIdx.x == 0 && blockIdx.y == 0);
+    const int b0 = 2 * blockIdx.z;
+    const bool act[2] = {os.outer_active[b0] != 0, b0 + 1 < nb && os.outer_active[b0 + 1] != 0};
+    if (!act[0] && !act[1]) return;
+    if (act[0]) tally_once(tl, blockIdx.x == 0 && blockIdx.y == 0);
+    if (act[1]) tally_once(tl, blockIdx.x == 0 && blockIdx.y == 0);
     const int nx = op.nx, nz = op.nz;
     const size_t N = (size_t)nx * nz;
-    const double2* xb = x + (size_t)b * N;
-    const float2* bb = bvec + (size_t)b * N;
-    float2* rb = r + (size_t)b * N;
     const int ix = blockIdx.x * TILE_X + threadIdx.x;
-    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * ROWS;
-    const double wf = op.omega[op.rhs_freq[b]];
-    const double w2 = wf * wf;
-    double acc_r = 0.0, acc_b = 0.0;
+    const int iz0 = (blockIdx.y * TILE_Y + threadIdx.y) * rows;
+    const int f0 = op.rhs_freq[b0], f1 = b0 + 1 < nb ? op.rhs_freq[b0 + 1] : f0;
+    double w2[2];
+    {
+        const double a = op.omega[f0], c = op.omega[f1];
+        w2[0] = a * a;
+        w2[1] = c * c;
+    }
+    const double d0 = 2.0 * ax + 2.0 * az;
+    double acc_r[2] = {0.0, 0.0}, acc_b[2] = {0.0, 0.0};
     if (ix < nx) {
-        for (int rr = 0; rr < ROWS; ++rr) {
-            int iz = iz0 + rr;
+        const double2 zero = make_double2(0.0, 0.0);
+        double2 xn[2], xc[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const double2* xb = x + (size_t)(b0 + q) * N + ix;
+            xn[q] = act[q] && iz0 > 0 && iz0 < nz ? xb[(size_t)(iz0 - 1) * nx] : zero;
+            xc[q] = act[q] && iz0 < nz ? xb[(size_t)iz0 * nx] : zero;
+        }
+        for (int rr = 0; rr < rows; ++rr) {
+            const int iz = iz0 + rr;
             if (iz >= nz) break;
-            size_t p = (size_t)iz * nx + ix;
-            double2 z0 = make_double2(0.0, 0.0);
-            double2 xc = xb[p];
-            double2 xw = ix > 0 ? xb[p - 1] : z0;
-            double2 xe = ix < nx - 1 ? xb[p + 1] : z0;
-            double2 xn = iz > 0 ? xb[p - nx] : z0;
-            double2 xs = iz < nz - 1 ? xb[p + nx] : z0;
-            float2 mg = op.mg[p];
-            double s = w2 * ((double)mg.x * (double)mg.x);
-            double ci = -s * (double)mg.y;                 // c = s (1 - i gamma)
-            double hx_ = ax * (2.0 * xc.x - xw.x - xe.x) + az * (2.0 * xc.x - xn.x - xs.x) - (s * xc.x - ci * xc.y);
-            double hy_ = ax * (2.0 * xc.y - xw.y - xe.y) + az * (2.0 * xc.y - xn.y - xs.y) - (s * xc.y + ci * xc.x);
-            float2 bv = bb[p];
-            double bx = bv.x, by = conj_b ? -(double)bv.y : (double)bv.y;
-            double rx = bx - hx_, ry = by - hy_;
-            rb[p] = make_float2((float)rx, (float)ry);
-            acc_r += rx * rx + ry * ry;
-            acc_b += bx * bx + by * by;
+            const size_t p = (size_t)iz * nx + ix;
+            const float2 mg = op.mg[p];
+            const double k = widen(mg.x), m = k * k, gam = widen(mg.y);
+            double s = 0.0, ci = 0.0, dd = 0.0;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (!act[q]) continue;
+                const double2* xb = x + (size_t)(b0 + q) * N + p;
+                const double2 xs = iz < nz - 1 ? xb[nx] : zero;
+                const double2 xw = ix > 0 ? xb[-1] : zero;
+                const double2 xe = ix < nx - 1 ? xb[1] : zero;
+                const float2 bv = bvec[(size_t)(b0 + q) * N + p];
+                if (q == 0 || f1 != f0 || !act[0]) {
+                    s = w2[q] * m;
+                    ci = s * gam;                                  // coefficient s (1 - i gamma)
+                    dd = d0 - s;
+                }
+                const double bx = widen(bv.x), by = widen(conj_b ? -bv.y : bv.y);
+                const double rx = fma(-ci, -xc[q].y, fma(-dd, xc[q].x, fma(az, xn[q].x + xs.x, fma(ax, xw.x + xe.x, bx))));
+                const double ry = fma(-ci, xc[q].x, fma(-dd, xc[q].y, fma(az, xn[q].y + xs.y, fma(ax, xw.y + xe.y, by))));
+                r[(size_t)(b0 + q) * N + p] = make_float2(narrow(rx), narrow(ry));
+                acc_r[q] = fma(rx, rx, fma(ry, ry, acc_r[q]));
+                if (FIRST) acc_b[q] = fma(bx, bx, fma(by, by, acc_b[q]));
+                xn[q] = xc[q];
+                xc[q] = xs;
+            }
         }
     }
-    __shared__ double2 sm[NWARPS];
-    double2 vals[1] = {make_double2(acc_r, acc_b)};
-    const int ntiles = gridDim.x * gridDim.y;
-    const int tile = blockIdx.y * gridDim.x + blockIdx.x;
-    double2* part = os.partials + (size_t)b * os.max_tiles;
-    bool last = reduce_block_last<1>(vals, 1, part + tile, os.counters + b, ntiles, sm);
-    if (last && threadIdx.x == 0 && threadIdx.y == 0) {
-        double2 t = sum_partials(part, ntiles, 1, 0);
-        os.rnorm2[b] = t.x;
-        if (first) os.bnorm2[b] = t.y;
+    __shared__ double2 sm[2][NWARPS];
+    __shared__ unsigned s_last[2];
+    const int tid = threadIdx.x + threadIdx.y * TILE_X, lane = tid & 31, warp = tid >> 5;
+    const int ntiles = gridDim.x * gridDim.y, tile = blockIdx.y * gridDim.x + blockIdx.x;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (!act[q]) continue;
+        const double a = warp_sum(acc_r[q]), c = FIRST ? warp_sum(acc_b[q]) : 0.0;
+        if (lane == 0) sm[q][warp] = make_double2(a, c);
+    }
+    __syncthreads();
+    if (tid < 2 && act[tid]) {
+        double2 t = make_double2(0.0, 0.0);
+        for (int w = 0; w < NWARPS; ++w) t = dadd(t, sm[tid][w]);
+        os.partials[(size_t)(b0 + tid) * ntiles + tile] = t;
+        __threadfence();
+        const unsigned n = atomicAdd(os.counters + b0 + tid, 1u);
+        s_last[tid] = n == (unsigned)ntiles - 1u ? 1u : 0u;
+        if (s_last[tid]) os.counters[b0 + tid] = 0u;
+    }
+    __syncthreads();
+    // the last block of an RHS sums the tiles (warp q for RHS b0 + q, lanes over the tiles in a fixed order)
+    if (warp < 2 && act[warp] && s_last[warp]) {
+        __threadfence();
+        double2 t = make_double2(0.0, 0.0);
+        for (int i = lane; i < ntiles; i += 32) t = dadd(t, __ldcg(os.partials + (size_t)(b0 + warp) * ntiles + i));
+        const double a = warp_sum(t.x), c = FIRST ? warp_sum(t.y) : 0.0;
+        if (lane == 0) {
+            os.rnorm2[b0 + warp] = a;
+            if (FIRST) os.bnorm2[b0 + warp] = c;
+        }
     }
 }
 
@@ -151,6 +266,14 @@ __global__ void zero_x_kernel(OuterState os, double2* x, size_t n) {
 
 int launch_apply_fine(const helm_ctx* c, const OpFine5& op, const float2* x, float2* y, int nb, const int* mask) {
     LaunchScope scope(c, K_APPLY);
+    // node pairs when the rows and the fields start on 16 bytes
+    if (op.nx % 2 == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0) {
+        const int xt = (op.nx / 2 + TILE_X - 1) / TILE_X, rows = arnoldi_rows(xt, op.nz, nb);
+        { apply_fine2_kernel<<<dim3(xt, (op.nz + TILE_Y * rows - 1) / (TILE_Y * rows), nb), dim3(TILE_X, TILE_Y), 0, c->stream>>>(
+            op, x, y, rows, mask, tally(c, K_APPLY, 16ull * op.nx * op.nz)); count_launch(); }
+        HELM_CK(cudaGetLastError());
+        return HELM_OK;
+    }
     { apply_fine_kernel<<<dim3((op.nx + 31) / 32, (op.nz + 7) / 8, nb), dim3(32, 8), 0, c->stream>>>(op, x, y, mask,
                                                                                                tally(c, K_APPLY, 16ull * op.nx * op.nz)); count_launch(); }
     HELM_CK(cudaGetLastError());
@@ -158,13 +281,17 @@ int launch_apply_fine(const helm_ctx* c, const OpFine5& op, const float2* x, flo
 }
 
 int launch_residual64(helm_ctx* c, const double2* x, const float2* b, float2* r, int nb, int conj_b, int first) {
-    OpFine5 op = fine_op(c, 0);
-    dim3 grid((c->nx + TILE_X - 1) / TILE_X, (c->nz + TILE_Y * ROWS - 1) / (TILE_Y * ROWS), nb);
+    const OpFine5 op = fine_op(c, 0);
+    // rows per thread as the Arnoldi kernels choose them: fewer on a small batch
+    const int xt = (c->nx + TILE_X - 1) / TILE_X, pairs = (nb + 1) / 2, rows = arnoldi_rows(xt, c->nz, pairs);
+    const dim3 grid(xt, (c->nz + TILE_Y * rows - 1) / (TILE_Y * rows), pairs);
+    const double ax = 1.0 / ((double)c->hx * c->hx), az = 1.0 / ((double)c->hz * c->hz);
+    const Tally tl = tally(c, K_RESIDUAL64, 32ull * c->nx * c->nz);
     LaunchScope scope(c, K_RESIDUAL64);
-    { residual64_kernel<<<grid, dim3(TILE_X, TILE_Y), 0, c->stream>>>(op, x, b, r, conj_b, first,
-                                                                    1.0 / ((double)c->hx * c->hx),
-                                                                    1.0 / ((double)c->hz * c->hz), c->outer,
-                                                                    tally(c, K_RESIDUAL64, 32ull * c->nx * c->nz)); count_launch(); }
+    if (first)
+        { residual64_kernel<true><<<grid, dim3(TILE_X, TILE_Y), 0, c->stream>>>(op, x, b, r, conj_b, nb, rows, ax, az, c->outer, tl); count_launch(); }
+    else
+        { residual64_kernel<false><<<grid, dim3(TILE_X, TILE_Y), 0, c->stream>>>(op, x, b, r, conj_b, nb, rows, ax, az, c->outer, tl); count_launch(); }
     HELM_CK(cudaGetLastError());
     return HELM_OK;
 }
