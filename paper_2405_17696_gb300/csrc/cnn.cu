@@ -1035,8 +1035,9 @@ int cnn_conv3x3_backward(const float* x0, int c0, const float* x1, int c1, int x
         auto* Wt = (__nv_bfloat16*)alloc((size_t)cp * 9 * npad * sizeof(__nv_bfloat16));
         float* fine = mode == 2 ? (float*)alloc(nout * cp * sizeof(float)) : nullptr;
         if (s) break;
-        ck(cudaMemset(target, 0, nin * cp * sizeof(float)));
-        if (!s) s = layer_dgrad(bg, npad, bw, cinp, part ? cp0 : 0, cp, mode, nb, hin, win, hout, wout, target, Wt,
+        GradOut go;
+        go.target = target;
+        if (!s) s = layer_dgrad(bg, npad, bw, cinp, part ? cp0 : 0, cp, mode, nb, hin, win, hout, wout, go, Wt,
                                 fine, err, nullptr, nullptr);
         ck(cudaDeviceSynchronize());
         if (s) break;

@@ -285,10 +285,23 @@ int layer_wgrad(const __nv_bfloat16* x0, int c0, const __nv_bfloat16* x1, int c1
                 int nb1, int nb, int hin, int win, int hout, int wout, int mode, const __nv_bfloat16* g, int npad,
                 int cout, int cin, float* dW, float* db, float** scratch, size_t* scratch_cap, int* err,
                 cudaStream_t st, const helm_ctx* prof_ctx);
-// target += W^T g for input channels off .. off + cp - 1 (tensor cores)
+// Where an input gradient goes.  target: FP32 [nb][hin][win][cp], added to with `accum`.  Or, with g, it
+// completes the gradient of the activation `mask`: prior (FP32, or nullptr) + it, masked, to g (BF16,
+// chunked) and, unmasked skips needing it, to res (FP32, added to with res_accum).
+struct GradOut {
+    float* target = nullptr;
+    int accum = 0;
+    const __nv_bfloat16* mask = nullptr;
+    const float* prior = nullptr;
+    __nv_bfloat16* g = nullptr;
+    float* res = nullptr;
+    int res_accum = 0;
+};
+// W^T g for input channels off .. off + cp - 1 (tensor cores); HELM_EUNSUPPORTED (nothing written) when
+// `out.g` is set and the layer runs on a kernel without that output
 int layer_dgrad(const __nv_bfloat16* g, int npad, const __nv_bfloat16* W, int cin_pad, int off, int cp, int mode,
-                int nb, int hin, int win, int hout, int wout, float* target, __nv_bfloat16* Wt, float* fine, int* err,
-                cudaStream_t st, const helm_ctx* prof_ctx);
+                int nb, int hin, int win, int hout, int wout, const GradOut& out, __nv_bfloat16* Wt, float* fine,
+                int* err, cudaStream_t st, const helm_ctx* prof_ctx);
 
 inline int check_conv_error(cnn_model* m, cudaStream_t st) {
     int h = 0;

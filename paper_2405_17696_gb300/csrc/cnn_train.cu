@@ -21,7 +21,7 @@
 #include <cmath>
 #include <string>
 #include <unordered_map>
-#include <unordered_set>
+#include <utility>
 #include <vector>
 
 #include <atomic>
@@ -38,7 +38,7 @@ namespace {
 // res_grad is given, res_grad += the FP32 masked gradient (same layout as G).
 __global__ void mask_to_bf16_kernel(const float* __restrict__ G, int cg, const __nv_bfloat16* __restrict__ y,
                                     int cy, int cpad, long long n, long long hw, __nv_bfloat16* __restrict__ out,
-                                    float* __restrict__ res_grad) {
+                                    float* __restrict__ res_grad, int res_accum) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n * cpad;
          i += (long long)gridDim.x * blockDim.x) {
         const long long p = i / cpad;
@@ -48,9 +48,23 @@ __global__ void mask_to_bf16_kernel(const float* __restrict__ G, int cg, const _
         if (c < cg) {
             v = G[p * cg + c];
             if (y && !(__bfloat162float(y[nc8(b, c, pix, cy, hw)]) > 0.0f)) v = 0.0f;
-            if (res_grad) res_grad[p * cg + c] += v;
+            if (res_grad) res_grad[p * cg + c] = res_accum ? res_grad[p * cg + c] + v : v;
         }
         out[nc8(b, c, pix, cpad, hw)] = __float2bfloat16_rn(v);
+    }
+}
+
+// The same for cg <= 8, cpad = 16, no mask and no skip (the output layer): a thread per pixel.
+__global__ void narrow_to_bf16_kernel(const float* __restrict__ G, int cg, long long hw, __nv_bfloat16* __restrict__ out) {
+    const long long b = blockIdx.y;
+    for (long long pix = blockIdx.x * (long long)blockDim.x + threadIdx.x; pix < hw;
+         pix += (long long)gridDim.x * blockDim.x) {
+        const float* g = G + (b * hw + pix) * cg;
+        uint4 o;
+        __nv_bfloat16* oh = reinterpret_cast<__nv_bfloat16*>(&o);
+        for (int j = 0; j < 8; ++j) oh[j] = __float2bfloat16_rn(j < cg ? g[j] : 0.0f);
+        *reinterpret_cast<uint4*>(out + nc8(b, 0, pix, 16, hw)) = o;
+        *reinterpret_cast<uint4*>(out + nc8(b, 8, pix, 16, hw)) = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -58,7 +72,7 @@ __global__ void mask_to_bf16_kernel(const float* __restrict__ G, int cg, const _
 // 16-byte loads and stores (grid.y = chunk, grid.z = image: no division per element).
 __global__ void mask_to_bf16_vec_kernel(const float* __restrict__ G, const __nv_bfloat16* __restrict__ y, int cy,
                                         int cpad, long long hw, __nv_bfloat16* __restrict__ out,
-                                        float* __restrict__ res_grad) {
+                                        float* __restrict__ res_grad, int res_accum) {
     const int c8 = blockIdx.y;
     const long long b = blockIdx.z;
     for (long long pix = blockIdx.x * (long long)blockDim.x + threadIdx.x; pix < hw;
@@ -76,7 +90,8 @@ __global__ void mask_to_bf16_vec_kernel(const float* __restrict__ G, const __nv_
         }
         if (res_grad) {
             float4* r4 = reinterpret_cast<float4*>(res_grad + p * cpad + 8 * c8);
-            float4 r0 = r4[0], r1 = r4[1];
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 r0 = res_accum ? r4[0] : z, r1 = res_accum ? r4[1] : z;
             r0.x += v[0]; r0.y += v[1]; r0.z += v[2]; r0.w += v[3];
             r1.x += v[4]; r1.y += v[5]; r1.z += v[6]; r1.w += v[7];
             r4[0] = r0;
@@ -100,29 +115,64 @@ __global__ void transpose_weights_kernel(const __nv_bfloat16* __restrict__ W, in
     }
 }
 
-// coarse[b][i][j][c] += sum of the 2x2 block of fine[b][2i..2i+1][2j..2j+1][c]
-__global__ void sumpool_accum_kernel(const float* __restrict__ fine, int nb, int h, int w, int c,
-                                     float* __restrict__ coarse) {
-    const long long total = (long long)nb * h * w * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = (int)(i % c);
-        long long r = i / c;
-        const int x = (int)(r % w);
-        r /= w;
-        const int y = (int)(r % h);
-        const int b = (int)(r / h);
-        const size_t W2 = 2 * (size_t)w;
-        const size_t base = (((size_t)b * 2 * h + 2 * y) * W2 + 2 * x) * c + ch;
-        coarse[i] += fine[base] + fine[base + c] + fine[base + W2 * c] + fine[base + W2 * c + c];
+// The 2x2 sums of fine [nb][2h][2w][c] (c a multiple of 8) as an input gradient (see GradOut): a thread per
+// coarse pixel and 8-channel chunk, 16-byte accesses; grid (pixels, chunks, images).
+__global__ void sumpool_grad_kernel(const float* __restrict__ fine, int h, int w, int c, GradOut o) {
+    const int c8 = blockIdx.y;
+    const long long b = blockIdx.z, hw = (long long)h * w;
+    const size_t row = 2 * (size_t)w * c;                     // a fine row
+    for (long long pix = blockIdx.x * (long long)blockDim.x + threadIdx.x; pix < hw;
+         pix += (long long)gridDim.x * blockDim.x) {
+        const int y = (int)(pix / w), x = (int)(pix - (long long)y * w);
+        const float* f = fine + (size_t)b * 4 * hw * c + 2 * y * row + 2 * (size_t)x * c + 8 * c8;
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float4 p0 = *reinterpret_cast<const float4*>(f + 4 * k);
+            const float4 p1 = *reinterpret_cast<const float4*>(f + c + 4 * k);
+            const float4 p2 = *reinterpret_cast<const float4*>(f + row + 4 * k);
+            const float4 p3 = *reinterpret_cast<const float4*>(f + row + c + 4 * k);
+            v[4 * k] = ((p0.x + p1.x) + p2.x) + p3.x;
+            v[4 * k + 1] = ((p0.y + p1.y) + p2.y) + p3.y;
+            v[4 * k + 2] = ((p0.z + p1.z) + p2.z) + p3.z;
+            v[4 * k + 3] = ((p0.w + p1.w) + p2.w) + p3.w;
+        }
+        const size_t at = ((size_t)b * hw + pix) * c + 8 * c8;
+        if (!o.g) {
+            float4* t4 = reinterpret_cast<float4*>(o.target + at);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float4 t = o.accum ? t4[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+                t4[k] = make_float4(t.x + v[4 * k], t.y + v[4 * k + 1], t.z + v[4 * k + 2], t.w + v[4 * k + 3]);
+            }
+            continue;
+        }
+        if (o.prior)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] += o.prior[at + j];
+        const size_t oc = nc8(b, 8 * c8, pix, c, hw);
+        const uint4 m = *reinterpret_cast<const uint4*>(o.mask + oc);
+        const __nv_bfloat16* mh = reinterpret_cast<const __nv_bfloat16*>(&m);
+        uint4 q;
+        __nv_bfloat16* qh = reinterpret_cast<__nv_bfloat16*>(&q);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (!(__bfloat162float(mh[j]) > 0.0f)) v[j] = 0.0f;
+            qh[j] = __float2bfloat16_rn(v[j]);
+        }
+        *reinterpret_cast<uint4*>(o.g + oc) = q;
+        if (o.res)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o.res[at + j] = o.res_accum ? o.res[at + j] + v[j] : v[j];
     }
 }
 
-// G_ctx[f] += sum over the samples b that use context image f (map(b) == f, or f = 0
+// G_ctx[f] (+)= sum over the samples b that use context image f (map(b) == f, or f = 0
 // when bcast == 1) of tmp[b], summed in the order of b: one thread per context element,
 // no atomics, so that the gradient is the same on every run
 __global__ void reduce_to_context_kernel(const float* __restrict__ tmp, long long per_image, int nb,
-                                         const int* __restrict__ map, int bcast, int nctx, float* __restrict__ gctx) {
+                                         const int* __restrict__ map, int bcast, int nctx, float* __restrict__ gctx,
+                                         int accum) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per_image * nctx;
          i += (long long)gridDim.x * blockDim.x) {
         const int f = (int)(i / per_image);
@@ -130,7 +180,7 @@ __global__ void reduce_to_context_kernel(const float* __restrict__ tmp, long lon
         float acc = 0.0f;
         for (int b = 0; b < nb; ++b)
             if ((bcast == 1 ? 0 : __ldg(map + b)) == f) acc += tmp[(long long)b * per_image + q];
-        gctx[i] += acc;
+        gctx[i] = accum ? gctx[i] + acc : acc;
     }
 }
 
@@ -401,14 +451,13 @@ int layer_wgrad(const __nv_bfloat16* x0, int c0, const __nv_bfloat16* x1, int c1
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_ECUDA;
 }
 
-// target += the input gradient W^T g of one input part (channels off .. off + cp - 1 of the
-// layer's padded input) on the tensor cores: 'same' -> same-grid convolution with
-// transposed, tap-flipped weights; 'down' -> the transpose-of-down mode; 'up' -> a
-// same-grid convolution on the fine grid, then a 2 x 2 sum.  target FP32 [nb][hin][win][cp];
-// Wt: scratch of cp x 9 x npad BF16; fine: scratch of nb x hout x wout x cp FP32 (mode 2).
+// The input gradient W^T g of one input part (channels off .. off + cp - 1 of the layer's padded input) on
+// the tensor cores, written as `out` says: 'same' -> same-grid convolution with transposed, tap-flipped
+// weights; 'down' -> the transpose-of-down mode; 'up' -> a same-grid convolution on the fine grid, then
+// a 2 x 2 sum.  Wt: scratch of cp x 9 x npad BF16; fine: scratch of nb x hout x wout x cp FP32 (mode 2).
 int layer_dgrad(const __nv_bfloat16* g, int npad, const __nv_bfloat16* W, int cin_pad, int off, int cp, int mode,
-                int nb, int hin, int win, int hout, int wout, float* target, __nv_bfloat16* Wt, float* fine, int* err,
-                cudaStream_t st, const helm_ctx* prof_ctx) {
+                int nb, int hin, int win, int hout, int wout, const GradOut& out, __nv_bfloat16* Wt, float* fine,
+                int* err, cudaStream_t st, const helm_ctx* prof_ctx) {
     {
         LaunchScope scope(prof_ctx, K_CNN_IO);
         { transpose_weights_kernel<<<256, 256, 0, st>>>(W, npad, cin_pad, off, cp, mode == 1 ? 0 : 1, Wt); count_launch(); }
@@ -416,15 +465,19 @@ int layer_dgrad(const __nv_bfloat16* g, int npad, const __nv_bfloat16* W, int ci
     ConvArgs ca;
     ca.x0 = g; ca.c0 = npad; ca.x1 = nullptr; ca.c1 = 0; ca.x1_bcast = 0; ca.x1_map = nullptr;
     ca.nb = nb; ca.w = Wt; ca.bias = nullptr; ca.res = nullptr; ca.npad = cp; ca.cstore = cp;
-    ca.relu = 0; ca.out_fp32 = 1; ca.accum = 1; ca.err = err;
+    ca.relu = 0; ca.out_fp32 = 1; ca.accum = 0; ca.err = err;
     ca.hin = hout; ca.win = wout;
     if (mode == 0 || mode == 1) {
-        ca.hout = hin; ca.wout = win; ca.mode = mode == 0 ? 0 : 3; ca.y = target;
+        ca.hout = hin; ca.wout = win; ca.mode = mode == 0 ? 0 : 3;
+        if (out.g) {
+            ca.y = out.g; ca.out_fp32 = 0;
+            ca.gmask = out.mask; ca.gprior = out.prior; ca.gres = out.res; ca.gres_accum = out.res_accum;
+        } else {
+            ca.y = out.target; ca.accum = out.accum;
+        }
         LaunchScope scope(prof_ctx, K_CONV);
         return launch_conv3x3(ca, st);
     }
-    const long long nout = (long long)nb * hout * wout;
-    if (cudaMemsetAsync(fine, 0, (size_t)nout * cp * sizeof(float), st) != cudaSuccess) return HELM_ECUDA;
     ca.hout = hout; ca.wout = wout; ca.mode = 0; ca.y = fine;
     int s;
     {
@@ -433,7 +486,9 @@ int layer_dgrad(const __nv_bfloat16* g, int npad, const __nv_bfloat16* W, int ci
     }
     if (s) return s;
     LaunchScope scope(prof_ctx, K_CNN_IO);
-    { sumpool_accum_kernel<<<1184, 256, 0, st>>>(fine, nb, hin, win, cp, target); count_launch(); }
+    const long long hw = (long long)hin * win;
+    const unsigned gx = (unsigned)std::max<long long>(1, std::min<long long>((hw + 255) / 256, std::max(1, 2432 / nb)));
+    { sumpool_grad_kernel<<<dim3(gx, (unsigned)(cp / 8), (unsigned)nb), 256, 0, st>>>(fine, hin, win, cp, out); count_launch(); }
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_ECUDA;
 }
 
@@ -512,47 +567,50 @@ class Backward {
    public:
     Backward(cnn_model* m, const helm_ctx* c, cudaStream_t st) : m_(m), c_(c), st_(st) {}
 
-    // gradient buffer of an activation (allocated and zeroed on first use)
-    float* grad_of(const void* act, size_t n) {
-        auto it = G_.find(act);
-        if (it != G_.end()) return it->second;
-        float* p = (float*)alloc(n * sizeof(float));
-        if (!p) return nullptr;
-        if (cudaMemsetAsync(p, 0, n * sizeof(float), st_) != cudaSuccess) ok_ = false;
-        G_[act] = p;
-        return p;
-    }
     void seed(const void* act, float* g) { G_[act] = g; }
 
     int run(const std::vector<TapeOp>& tape, int nctx) {
-        std::unordered_set<const void*> produced;
-        for (const TapeOp& op : tape) produced.insert(op.y);
+        // The op that produces each activation, and where the backward pass adds the last part of its
+        // gradient: (op, slot), slots 0 (its skip), 1, 2 (its inputs) of ops from the last to the first.
+        std::unordered_map<const void*, int> producer;
+        std::unordered_map<const void*, std::pair<int, int>> last;
+        for (int k = 0; k < (int)tape.size(); ++k) producer[tape[k].y] = k;
+        for (int k = (int)tape.size() - 1; k >= 0; --k) {
+            const void* in[3] = {tape[k].res, tape[k].x0, tape[k].x1};
+            for (int s = 0; s < 3; ++s)
+                if (in[s]) last[in[s]] = {k, s};
+        }
+        std::unordered_map<const void*, __nv_bfloat16*> ready;   // masked BF16 gradients written by a consumer
         for (int k = (int)tape.size() - 1; k >= 0 && ok_; --k) {
             const TapeOp& op = tape[k];
-            auto it = G_.find(op.y);
-            if (it == G_.end()) continue;
-            const float* Gy = it->second;
             const Layer& L = m_->layers[op.layer];
             const bool is_out = L.cout < 16;   // the 2-channel output layer (FP32 output, no activation)
             const long long nout = (long long)op.nb * op.hout * op.wout;
-            const int cg = is_out ? L.cout : L.npad;
-            __nv_bfloat16* g = (__nv_bfloat16*)alloc((size_t)nout * L.npad * sizeof(__nv_bfloat16));
-            float* rg = op.res ? grad_of(op.res, (size_t)nout * L.npad) : nullptr;
-            if (!ok_) break;
-            {
+            const __nv_bfloat16* g = nullptr;
+            auto rit = ready.find(op.y);
+            if (rit != ready.end()) {
+                g = rit->second;
+            } else {
+                auto it = G_.find(op.y);
+                if (it == G_.end()) continue;
+                const float* Gy = it->second;
+                const int cg = is_out ? L.cout : L.npad;
+                __nv_bfloat16* gw = (__nv_bfloat16*)alloc((size_t)nout * L.npad * sizeof(__nv_bfloat16));
+                const int had = op.res && G_.count(op.res) ? 1 : 0;
+                float* rg = op.res ? grad_of(op.res, (size_t)nout * L.npad) : nullptr;
+                if (!ok_) break;
                 LaunchScope scope(c_, K_CNN_IO);
                 const __nv_bfloat16* ymask = L.relu ? (const __nv_bfloat16*)op.y : nullptr;
+                const long long hw = (long long)op.hout * op.wout;
+                const long long bx = std::max<long long>(1, std::min<long long>((hw + 255) / 256, 1184 / op.nb));
                 if (cg == L.npad && cg % 8 == 0)
-                {
-                    const long long hw = (long long)op.hout * op.wout;
-                    const long long bx = std::max<long long>(1, std::min<long long>((hw + 255) / 256, 1184 / op.nb));
-                    mask_to_bf16_vec_kernel<<<dim3((unsigned)bx, (unsigned)(cg / 8), (unsigned)op.nb), 256, 0, st_>>>(
-                        Gy, ymask, L.npad, L.npad, hw, g, rg);
-                    count_launch();
-                }
+                    { mask_to_bf16_vec_kernel<<<dim3((unsigned)bx, (unsigned)(cg / 8), (unsigned)op.nb), 256, 0, st_>>>(
+                        Gy, ymask, L.npad, L.npad, hw, gw, rg, had); count_launch(); }
+                else if (cg <= 8 && L.npad == 16 && !ymask && !rg)
+                    { narrow_to_bf16_kernel<<<dim3((unsigned)bx, (unsigned)op.nb), 256, 0, st_>>>(Gy, cg, hw, gw); count_launch(); }
                 else
-                    { mask_to_bf16_kernel<<<1184, 256, 0, st_>>>(Gy, cg, ymask, L.npad, L.npad, nout,
-                                                              (long long)op.hout * op.wout, g, rg); count_launch(); }
+                    { mask_to_bf16_kernel<<<1184, 256, 0, st_>>>(Gy, cg, ymask, L.npad, L.npad, nout, hw, gw, rg, had); count_launch(); }
+                g = gw;
             }
             // weight and bias gradient
             {
@@ -568,31 +626,57 @@ class Backward {
             for (int part = 0; part < 2 && ok_; ++part) {
                 const __nv_bfloat16* x = part ? op.x1 : op.x0;
                 const int cp = part ? op.c1 : op.c0;
-                if (!x || cp == 0 || !produced.count(x)) continue;
+                auto pit = x && cp ? producer.find(x) : producer.end();
+                if (pit == producer.end()) continue;
                 const int shared = part == 1 && op.x1_bcast != 0;
                 const long long nin = (long long)op.nb * op.hin * op.win;
                 __nv_bfloat16* Wt = (__nv_bfloat16*)alloc((size_t)cp * 9 * L.npad * sizeof(__nv_bfloat16));
-                if (!ok_) break;
-                float* target;
-                if (shared) {
-                    target = (float*)alloc((size_t)nin * cp * sizeof(float));
-                    if (target) cudaMemsetAsync(target, 0, (size_t)nin * cp * sizeof(float), st_);
-                } else {
-                    target = grad_of(x, (size_t)nin * cp);
-                }
                 float* fine = L.mode == 2 ? (float*)alloc((size_t)nout * cp * sizeof(float)) : nullptr;
-                if (!ok_ || !target) { ok_ = false; break; }
-                const int s = layer_dgrad(g, L.npad, L.w, L.cin_pad, part ? op.c0 : 0, cp, L.mode, op.nb, op.hin,
-                                          op.win, op.hout, op.wout, target, Wt, fine, m_->err, st_, c_);
-                if (s != HELM_OK) { ok_ = false; break; }
+                if (!ok_) break;
+                auto dgrad = [&](const GradOut& o) {
+                    return layer_dgrad(g, L.npad, L.w, L.cin_pad, part ? op.c0 : 0, cp, L.mode, op.nb, op.hin, op.win,
+                                       op.hout, op.wout, o, Wt, fine, m_->err, st_, c_);
+                };
                 if (shared) {
+                    GradOut o;
+                    o.target = (float*)alloc((size_t)nin * cp * sizeof(float));
+                    if (!ok_ || dgrad(o) != HELM_OK) { ok_ = false; break; }
                     const long long per = (long long)op.hin * op.win * cp;
+                    const int had = G_.count(x) ? 1 : 0;
                     float* gctx = grad_of(x, (size_t)(op.x1_bcast == 1 ? 1 : nctx) * per);
                     if (!gctx) { ok_ = false; break; }
                     LaunchScope scope(c_, K_CNN_IO);
-                    { reduce_to_context_kernel<<<1184, 256, 0, st_>>>(target, per, op.nb, op.zmap, op.x1_bcast,
-                                                                    op.x1_bcast == 1 ? 1 : nctx, gctx); count_launch(); }
+                    { reduce_to_context_kernel<<<1184, 256, 0, st_>>>(o.target, per, op.nb, op.zmap, op.x1_bcast,
+                                                                    op.x1_bcast == 1 ? 1 : nctx, gctx, had); count_launch(); }
+                    continue;
                 }
+                // The last part of x's gradient completes it: the kernel that computes it writes the masked
+                // BF16 operand of the producing layer (and the FP32 copy its skip adds up) itself.
+                const TapeOp& pop = tape[pit->second];
+                const Layer& P = m_->layers[pop.layer];
+                int s = HELM_EUNSUPPORTED;
+                if (last[x] == std::make_pair(k, part + 1) && P.relu && P.npad == cp && P.cout >= 16) {
+                    GradOut o;
+                    auto gi = G_.find(x);
+                    o.prior = gi == G_.end() ? nullptr : gi->second;
+                    o.mask = x;
+                    o.g = (__nv_bfloat16*)alloc((size_t)nin * cp * sizeof(__nv_bfloat16));
+                    o.res_accum = pop.res && G_.count(pop.res) ? 1 : 0;
+                    const bool fresh_res = pop.res && !o.res_accum;
+                    if (pop.res) o.res = grad_of(pop.res, (size_t)nin * cp);
+                    if (!ok_) break;
+                    s = dgrad(o);
+                    if (s == HELM_OK) ready[x] = o.g;
+                    else if (s == HELM_EUNSUPPORTED && fresh_res) G_.erase(pop.res);   // (nothing was written)
+                }
+                if (s == HELM_EUNSUPPORTED) {
+                    GradOut o;
+                    o.accum = G_.count(x) ? 1 : 0;
+                    o.target = grad_of(x, (size_t)nin * cp);
+                    if (!ok_) break;
+                    s = dgrad(o);
+                }
+                if (s != HELM_OK) { ok_ = false; break; }
             }
         }
         if (cudaGetLastError() != cudaSuccess) ok_ = false;
@@ -600,6 +684,14 @@ class Backward {
     }
 
    private:
+    // FP32 gradient buffer of an activation; new ones are written before they are added to
+    float* grad_of(const void* act, size_t n) {
+        auto it = G_.find(act);
+        if (it != G_.end()) return it->second;
+        float* p = (float*)alloc(n * sizeof(float));
+        if (p) G_[act] = p;
+        return p;
+    }
     // scratch of the backward pass from the model's arena (the k-th request of a pass reuses
     // the k-th buffer of the previous step: one training step's pass has the same sequence)
     void* alloc(size_t bytes) {

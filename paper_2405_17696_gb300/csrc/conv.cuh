@@ -42,7 +42,7 @@ struct ConvArgs {
     const __nv_bfloat16* w;    // [npad][9][c0 + c1]
     const __nv_bfloat16* wup = nullptr;   // mode 2: the phase-merged weights [npad][16][c0 + c1]
                                           // (up_merged_index), which the tensor-map kernel needs
-    const float* bias;         // [npad]
+    const float* bias;         // [npad], or nullptr: none
     const __nv_bfloat16* res;  // [nb][npad/8][hout][wout][8] added before the activation, or nullptr
     void* y;                   // bf16 [nb][npad/8][hout][wout][8], or fp32 [nb][hout][wout][cstore]
     int npad;                  // N of the MMA: 16, 32, 64 or 128
@@ -51,8 +51,16 @@ struct ConvArgs {
     int out_fp32;
     int accum;                 // with out_fp32: y += result (no bias, no activation)
     int* err;                  // set to 1 when a bounded wait expires
+    // Gradient output (the backward pass; only in the tensor-map kernel, see launch_conv3x3): with
+    // gmask the result v (+ gprior) is the whole gradient of the activation gmask, and y receives
+    // bf16(v . [gmask > 0]), gres the same in FP32 (added to it with gres_accum).
+    const __nv_bfloat16* gmask = nullptr;   // [nb][npad/8][hout][wout][8]
+    const float* gprior = nullptr;          // [nb][hout][wout][npad], or nullptr
+    float* gres = nullptr;                  // [nb][hout][wout][npad], or nullptr
+    int gres_accum = 0;
 };
 
+// HELM_EUNSUPPORTED (nothing launched) for a gradient output (gmask) that only the gather kernel could take.
 int launch_conv3x3(const ConvArgs& a, cudaStream_t st);
 // layers through TMA-staged halo tiles (k_conv_tma.cu); HELM_EINVAL = not launched.
 // narrow: 0 plain; 1, 16-channel same-grid layers take the column-taps-in-N variant;

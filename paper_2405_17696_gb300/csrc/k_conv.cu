@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(NT) conv3x3_tc_kernel(ConvArgs a) {
             float v[16];
             tc::tmem_ld16(trow + col0, v);
             if (!valid) continue;
-            if (!a.accum) {
+            if (!a.accum && a.bias) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] += __ldg(a.bias + col0 + i);
             }
@@ -289,7 +289,7 @@ int launch_conv3x3(const ConvArgs& a, cudaStream_t st) {
         return HELM_EINVAL;
     }
     if (a.nb < 1 || a.hin < 1 || a.win < 1 || a.mode < 0 || a.mode > 3 || (a.accum && !a.out_fp32) ||
-        (!a.accum && !a.bias)) {
+        (a.gmask && a.out_fp32)) {
         set_error("conv3x3: bad shape or mode");
         return HELM_EINVAL;
     }
@@ -305,6 +305,7 @@ int launch_conv3x3(const ConvArgs& a, cudaStream_t st) {
             return t;
         }
     }
+    if (a.gmask) return HELM_EUNSUPPORTED;
     ++g_launch_gather;
     int ck = 64;
     if (a.c0 % 64 || (a.c1 && a.c1 % 64)) ck = 32;

@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
     constexpr int EPI_WARPS = epi_warps(MODE);
     constexpr int EPI = 32 * EPI_WARPS;             // epilogue threads
     const int tid = threadIdx.x, warp = tid >> 5;
-    if (tid < a.npad) bias_s[tid] = a.accum ? 0.0f : __ldg(a.bias + tid);
+    if (tid < a.npad) bias_s[tid] = a.accum || !a.bias ? 0.0f : __ldg(a.bias + tid);
     if (warp == 0) {
         tc::tmem_alloc(&tmem_base, g.tmem_cols);
         tc::tmem_relinquish();
@@ -529,6 +529,41 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
             if (a.relu) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) vv[i] = fmaxf(vv[i], 0.0f);
+            }
+            if (a.gmask) {
+                // the gradient of an activation: what is there already, the ReLU mask, the skip's FP32 copy
+                if (a.gprior) {
+                    const float4* q4 = reinterpret_cast<const float4*>(a.gprior + (size_t)p * a.npad + n0);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 t = __ldg(q4 + q);
+                        vv[4 * q] += t.x;
+                        vv[4 * q + 1] += t.y;
+                        vv[4 * q + 2] += t.z;
+                        vv[4 * q + 3] += t.w;
+                    }
+                }
+                const uint4 m0 = __ldg(reinterpret_cast<const uint4*>(a.gmask + o0));
+                const uint4 m1 = __ldg(reinterpret_cast<const uint4*>(a.gmask + o0 + plane_out));
+                const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
+                const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (!(__bfloat162float(mb0[i]) > 0.0f)) vv[i] = 0.0f;
+                    if (!(__bfloat162float(mb1[i]) > 0.0f)) vv[8 + i] = 0.0f;
+                }
+                if (a.gres) {
+                    float4* r4 = reinterpret_cast<float4*>(a.gres + (size_t)p * a.npad + n0);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float4 t = a.gres_accum ? r4[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        t.x += vv[4 * q];
+                        t.y += vv[4 * q + 1];
+                        t.z += vv[4 * q + 2];
+                        t.w += vv[4 * q + 3];
+                        r4[q] = t;
+                    }
+                }
             }
             if (a.out_fp32) {
                 float* yo = reinterpret_cast<float*>(a.y) + (size_t)p * a.cstore;
@@ -1232,8 +1267,8 @@ std::atomic<int> g_tuning{0};
 
 std::string shape_key(const ConvArgs& a) {
     char buf[160];
-    std::snprintf(buf, sizeof buf, "%d:%d:%d:%d:%d:%d:%d:%d:%d:%d:%d:%d", a.mode, a.c0, a.c1, a.x1_bcast,
-                  a.x1_map ? 1 : 0, a.hin, a.win, a.npad, a.res ? 1 : 0, a.out_fp32, a.accum, a.relu);
+    std::snprintf(buf, sizeof buf, "%d:%d:%d:%d:%d:%d:%d:%d:%d:%d:%d:%d:%d", a.mode, a.c0, a.c1, a.x1_bcast,
+                  a.x1_map ? 1 : 0, a.hin, a.win, a.npad, a.res ? 1 : 0, a.out_fp32, a.accum, a.relu, a.bias ? 1 : 0);
     return buf;
 }
 
@@ -1346,7 +1381,7 @@ int launch_conv3x3_tma(const ConvArgs& a, cudaStream_t st, int narrow) {
         if (it != g_tuned.end())
             t = it->second;
         else   // a layer is re-run while tuning only if that leaves its result unchanged
-            tune = g_tuning.load() && !a.accum && a.y != a.x0 && a.y != a.x1 && a.y != a.res;
+            tune = g_tuning.load() && !a.accum && !a.gres && a.y != a.x0 && a.y != a.x1 && a.y != a.res;
     }
     return tune ? tune_and_launch(a, st, key, t) : launch_cfg(a, st, t);
 }

@@ -278,12 +278,28 @@ __global__ void __launch_bounds__(256) bias_partial_kernel(const __nv_bfloat16* 
     const int c8 = blockIdx.y, seg = blockIdx.x;
     const long long p0 = (long long)seg * seg_len, p1 = min(npix, p0 + seg_len);
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (long long p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        const long long b = p / hw, pix = p - b * hw;
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(gr + nc8(b, 8 * c8, pix, npad, hw)));
-        const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v);
+    // image and pixel advance as counters (a 64-bit division per pixel cost more than its load), four loads in flight
+    long long p = p0 + threadIdx.x;
+    long long b = p / hw, pix = p - b * hw;
+    while (p < p1) {
+        uint4 v[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(h[j]);
+        for (int k = 0; k < 4; ++k) {
+            v[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (p < p1) v[k] = __ldg(reinterpret_cast<const uint4*>(gr + nc8(b, 8 * c8, pix, npad, hw)));
+            p += blockDim.x;
+            pix += blockDim.x;
+            while (pix >= hw) {
+                pix -= hw;
+                ++b;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&v[k]);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(h[j]);
+        }
     }
     __shared__ float red[256][9];
 #pragma unroll
