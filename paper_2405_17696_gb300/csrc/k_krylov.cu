@@ -103,9 +103,9 @@ __device__ void givens_step(const KState& st, int b, double n2, double inv_est, 
     if (!finite || tiny || est <= tol || cap || J + 1 >= st.k) st.active[b] = 0;
 }
 
-// (With FP64 shuffles the J + 2 sums of a block took some 7 us; at J = 9, 512 x 256 and 192 right-hand
-// sides on one GB300 the pass took 463 us with them and takes 310, 302 MB per basis vector at 7.8 TB/s
-// counting what L2 keeps; 20 us and 10 for one right-hand side of 160 x 160, with one row per thread.)
+// The block sums have no FP64 shuffles: those run at two lanes per SM and cycle, and a block has J + 2 sums.
+// Measured on one GB300 at J = 9, with them and without: 463 and 310 us for 512 x 256 and 192 right-hand
+// sides, 20 and 10 us for one right-hand side of 160 x 160 (there with one row per thread as well).
 // The block's part of the inner products acc[i] = <v~_i, w>, i <= J, acc[J + 1] = ||w||^2; the last block of
 // the RHS scales them to column J of the Hessenberg matrix and estimates ||w'||.
 template <int J>
@@ -301,7 +301,8 @@ __global__ void normalize_v0_kernel(KState st, float2* __restrict__ v0, size_t n
 }
 
 // Back substitution R y = g (FP64), one warp per RHS: lane i carries row i, and the
-// reciprocals of the diagonal are taken by all lanes at once.
+// reciprocals of the diagonal are taken by all lanes at once.  A serial chain of FP64 operations bounds
+// it: 160 x 160, one right-hand side, one GB300: 23.1 us with a thread per RHS, 5.7 us.
 __global__ void lsq_kernel(KState st, int nb) {
     const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (b >= nb) return;

@@ -29,7 +29,7 @@ __global__ void apply_fine_kernel(OpFine5 op, const float2* __restrict__ x, floa
 // field is read about once (the neighbours' columns come from L1) with 16-byte accesses.  The rounded
 // operations are those of OpFine5::apply in apply_fine_kernel, spelled out: the training pairs made
 // from H x do not depend on which kernel made it.  512 x 256, 192 fields, one GB300:
-// 115 -> 68 us (403 MB: 5.9 TB/s).
+// 115 -> 68 us (403 MB: 5.9 TB/s), 135 -> 96 us with the call's host part.
 __global__ void __launch_bounds__(NTHREADS) apply_fine2_kernel(OpFine5 op, const float2* __restrict__ x,
                                                                float2* __restrict__ y, int rows, const int* mask,
                                                                Tally tl) {
@@ -100,7 +100,7 @@ __device__ __forceinline__ float narrow(double d) {
 //   r = b + ax (xw + xe) + az (xn + xs) - (2 ax + 2 az - w^2 m) xc - i (w^2 m gamma) xc
 // with w^2 m and its products shared by a thread's two right-hand sides of one frequency, against
 // 34 in the order the operator is written, its conversions included.  512 x 256, 192 right-hand
-// sides, one GB300: 1.92 -> 1.31 ms a call, 1.47 -> 0.90 ms inside a solve.
+// sides, one GB300: 1.93 -> 1.32 ms a call, 1.47 -> 0.90 ms inside a solve.
 template <bool FIRST>
 __global__ void __launch_bounds__(NTHREADS) residual64_kernel(OpFine5 op, const double2* __restrict__ x,
                                                               const float2* __restrict__ bvec,
