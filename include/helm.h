@@ -489,7 +489,8 @@ void cnn_autotune_reset(void);
  * row-taps-in-N variant for 16- and 32-channel ones, narrow = 3 the tiling with one
  * accumulator buffer of up to 512 TMEM columns (any mode; an autotuner candidate),
  * narrow = 4 an up layer with a tile per output row parity (cnn_set_conv_upsplit; 2
- * parities per tile, tiles counted per parity), narrow = 5 both of the last two.
+ * parities per tile, tiles counted per parity), narrow = 5 both of the last two,
+ * narrow = 6 the tiling of a default launch (mode used 5 or 0).
  * out19 = {tiles,
  * tile width, tile rows, staged row pitch, M blocks per parity, parities,
  * parity sub-planes, plane bytes, parity stride bytes, weight bytes, stage

@@ -35,6 +35,16 @@
 //    warp: two shuffles).  Each staged pixel is read by 3 MMAs instead of 9; the rows 6
 //    and 7 of each group are computed and dropped.  Accumulators live in a ring of
 //    per-M-block TMEM slots, so that a tile's size is not bounded by TMEM.
+//  5 (same grid as mode 0, same sums in the same order) an M block is one staged row (pitch
+//    tw + 2 <= 128, lanes >= tw dropped) and the accumulators of a tile's output rows lie side
+//    by side in TMEM, the last row first.  Staged row b adds to output rows b - 2, b - 1 and b
+//    with tap rows 2, 1 and 0: adjacent columns, so that one MMA with N = 3 npad per column shift
+//    serves all three (N = npad or 2 npad at the tile's ends).  A pixel is read by 3 MMAs instead
+//    of 9, and an output row still sums (group, dy, dx) in mode 0's order, bit for bit.  One MMA
+//    of zeros clears the tile's columns, since every other one adds to rows in progress.  Mode 0
+//    at 32 -> 16 channels spends 76 % of the cycles on operand reads; 1024 x 512, 32 images, one
+//    GB300, mode 0 and mode 5: 344 and 305 us for one layer of 16 channels;
+//    the 29 layers of a network pass took 7.41 ms and take 7.17.
 //  6 (16 or 32 output channels, same grid as mode 0) the three tap rows in N: an M block is
 //    one staged row (pitch tw + 2 <= 128, lanes >= tw dropped) and per 16-channel group takes
 //    three MMAs, one per column shift dx, computing D[b][x][(dy, o)] for N = 3 npad.  Output
@@ -93,6 +103,7 @@ constexpr size_t RING_BUDGET_RT32 = 200 * 1024;  // mode 6, 32 channels: one CTA
 constexpr int ROWS_RT_MAX = 32;                 // mode 6: output rows per tile at most
 constexpr int RT_CHUNK = 4;                     // mode 6: staged rows per commit at most (a commit
                                                 // costs about as much as several MMAs)
+constexpr int ZERO_BYTES = 256 * 32;            // mode 5: zero operands of the clearing MMA
 constexpr long long WAIT_LIMIT = 1ll << 22;     // polls of try_wait before a wait gives up
 // No padding after a plane: the last M block of a packed tile may read up to
 // 2 pitches + 130 pixels past its plane's staged pixels, which lands in the next
@@ -119,6 +130,7 @@ struct Geometry {
     int nslot, slot_cols;    // modes 4 and 6: TMEM slots (an M block / a staged row each) and their columns
     int nbuf;                // modes 0-3: TMEM accumulator buffers (2: the epilogue drains one while
                              // the MMAs fill the other; 1: twice the M blocks per tile)
+    int nzero;               // mode 5: columns that the clearing MMA writes (rows * npad)
     int nwg;                 // mode 6: epilogue warpgroups that take output rows
     int chunk;               // mode 6: staged rows per commit
     int psplit;              // mode 2: a tile computes one output row parity py (nph = 2: px), the
@@ -188,11 +200,18 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
     __shared__ float bias_s[128];
+    // mode 5: both operands of the clearing MMA (A 128 rows, B up to 256 rows of 16 zeros)
+    __shared__ __align__(128) unsigned char zeros[MODE == 5 ? ZERO_BYTES : 16];
 
     constexpr int EPI_WARPS = epi_warps(MODE);
     constexpr int EPI = 32 * EPI_WARPS;             // epilogue threads
     const int tid = threadIdx.x, warp = tid >> 5;
     if (tid < a.npad) bias_s[tid] = a.accum || !a.bias ? 0.0f : __ldg(a.bias + tid);
+    if constexpr (MODE == 5) {
+        for (int i = tid * 16; i < ZERO_BYTES; i += (int)blockDim.x * 16)
+            *reinterpret_cast<uint4*>(zeros + i) = make_uint4(0u, 0u, 0u, 0u);
+        tc::fence_proxy_async_smem();   // the MMAs read them through the async proxy
+    }
     if (warp == 0) {
         tc::tmem_alloc(&tmem_base, g.tmem_cols);
         tc::tmem_relinquish();
@@ -274,9 +293,9 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                     }
                 }
                 unsigned char* ws = st + wofs;
-                if (MODE == 4 || MODE == 6) {
+                if (MODE == 4 || MODE == 5 || MODE == 6) {
                     // mode 4 [dy][half][dx][npad][8]: the B operand of tap row dy is 3 npad rows (dx, o);
-                    // mode 6 [dx][half][dy][npad][8]: the B operand of column shift dx is 3 npad rows (dy, o)
+                    // modes 5 and 6 [dx][half][dy][npad][8]: the B operand of column shift dx is 3 npad rows (dy, o)
                     tc::tma_load_5d(ws, &tm_w, 0, 0, 0, 2 * gi, 0, &full[s]);
                 } else if (g.w4) {
                     // split parities: the 8 merged taps of the tile's row parity
@@ -426,6 +445,59 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                 if (leader)
                     for (int gi = 0; gi < G; ++gi) tc::mma_commit(&empty[(j + gi) % g.ns]);
                 j += G;
+            }
+        } else if constexpr (MODE == 5) {
+            // output row r of the tile accumulates in columns (rows - 1 - r) npad of the buffer;
+            // staged row b and column shift dx: rows r = b - t for the tap rows t that exist
+            const uint64_t bdesc5 = tc::smem_desc(0u, 3u * wplane, 128);   // K halves 3 npad rows apart
+            const uint32_t b5_lo = (uint32_t)bdesc5, b5_hi = (uint32_t)(bdesc5 >> 32);
+            const uint32_t dx_b16 = (6u * wplane) >> 4;                    // B of one column shift
+            const uint32_t id1 = tc::idesc_bf16_f32(128, a.npad), id2 = tc::idesc_bf16_f32(128, 2 * a.npad),
+                           id3 = tc::idesc_bf16_f32(128, 3 * a.npad), idz = tc::idesc_bf16_f32(128, g.nzero);
+            const uint64_t az = tc::smem_desc(tc::smem_u32(zeros), 128 * 16, 128);
+            const uint64_t bz = tc::smem_desc(tc::smem_u32(zeros), (uint32_t)g.nzero * 16, 128);
+            const int R = g.rows;
+            int s = 0, wraps = 0;   // j % ns and j / ns as counters
+            for (int k = 0; k < ntiles && ok; ++k) {
+                const int acc = g.nbuf == 2 ? (k & 1) : 0;
+                const int ause = g.nbuf == 2 ? (k >> 1) : k;
+                const bool t_ok = ause == 0 || wait_bar(&tempty[acc], (uint32_t)((ause - 1) & 1), abort_v, 32);
+                if (!__all_sync(0xffffffffu, t_ok)) { ok = false; break; }
+                tc::tc_fence_after_sync();
+                const uint32_t dbase = tmem + (uint32_t)acc * g.acc_cols;
+                if (leader) tc::mma_bf16(dbase, az, bz, idz, 0u);
+                for (int gi = 0; gi < G; ++gi, ++j) {
+                    if (gi > 0 || k > 0)
+                        if (++s == g.ns) {
+                            s = 0;
+                            ++wraps;
+                        }
+                    const bool f_ok = wait_bar(&full[s], (uint32_t)(wraps & 1), abort_v, 32);
+                    if (!__all_sync(0xffffffffu, f_ok)) { ok = false; break; }
+                    tc::tc_fence_after_sync();
+                    const uint32_t a16 = (tc::smem_u32(smem + (size_t)s * g.stage) & 0x3FFFFu) >> 4;
+                    const uint32_t b_s = b5_lo + a16 + ((uint32_t)wofs >> 4);
+                    uint32_t a_b = a_lo0 + a16;
+                    for (int b = 0; b < R + 2; ++b, a_b += (uint32_t)g.pw) {
+                        const int t0 = b < R ? 0 : b - R + 1;          // first and last tap row in use
+                        const int t1 = b < 2 ? b : 2;
+                        const uint32_t d = dbase + (uint32_t)((R - 1 - b + t0) * a.npad);
+                        const uint32_t b_t = b_s + (uint32_t)(t0 * a.npad);   // 16 bytes per row of B
+                        const uint32_t id = t1 - t0 == 2 ? id3 : (t1 - t0 == 1 ? id2 : id1);
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx) {
+                            if (leader) {
+                                const uint64_t ad = ((uint64_t)a_hi << 32) | (a_b + (uint32_t)dx);
+                                const uint64_t bd = ((uint64_t)b5_hi << 32) | (b_t + (uint32_t)dx * dx_b16);
+                                tc::mma_bf16(d, ad, bd, id, 1u);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    if (leader) tc::mma_commit(&empty[s]);
+                }
+                __syncwarp();
+                if (ok && leader) tc::mma_commit(&tfull[acc]);
             }
         } else {
             int s = 0, wraps = 0;   // j % ns and j / ns as counters
@@ -721,8 +793,11 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                 const size_t img_base = (size_t)b * (size_t)(a.npad >> 3) * (size_t)hw_out * 8;
                 int m_prev = -4, yy = 0, xx = 0;
                 for (int bi = wg; bi < nblk; bi += 2) {
-                    const int ph = bi / g.mb, m = bi - ph * g.mb;
-                    if (m != m_prev + 2) {
+                    const int ph = MODE == 5 ? 0 : bi / g.mb, m = bi - ph * g.mb;
+                    if (MODE == 5) {
+                        yy = bi;      // a block is an output row
+                        xx = row;
+                    } else if (m != m_prev + 2) {
                         const int q = m * 128 + row;
                         yy = q / g.pw;
                         xx = q - yy * g.pw;
@@ -745,7 +820,7 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                     const long long pix = (long long)oy * a.wout + ox;
                     const size_t ob = img_base + (size_t)pix * 8;   // channel 0 of this pixel
                     const long long p = (long long)b * hw_out + pix;
-                    const uint32_t tcol = dbase + (uint32_t)(bi * a.npad);
+                    const uint32_t tcol = dbase + (uint32_t)((MODE == 5 ? g.rows - 1 - bi : bi) * a.npad);
                     if (a.npad == 16) {
                         float v[16];
                         tc::tmem_ld16(tcol, v);
@@ -906,6 +981,7 @@ std::atomic<int> g_rows_cap{0};   // tile-height limit set by cnn_set_conv_tilin
 // (mode 4, 16 output channels); narrow = 2, the row-taps-in-N kernel (mode 6, 16 or 32).
 struct TileCfg {
     int rows_cap = 0, stage_kb = 0, ring_kb = 0, narrow = 0;
+    int plain = 0;    // same-grid layers: mode 0 also where mode 5 takes fewer cycles (see rowsum_pays)
     int single = 0;   // modes 0-3: one accumulator buffer of up to 512 TMEM columns
     int upsplit = 0;  // mode 2: a tile per output row parity (half the weights per stage, twice the rows)
 };
@@ -920,8 +996,7 @@ int g_last_launch[6] = {0, 0, 0, 0, 0, 0};   // grid, CTAs per SM, CTAs register
 // Tile plan; .tiles = 0 when the layer does not fit this kernel.
 Geometry plan(const ConvArgs& a, const TileCfg& t) {
     Geometry g{};
-    const int mode = a.mode;
-    if (mode == 6) {
+    if (a.mode == 6) {
         // same grid, 16 or 32 output channels, tap rows in N (see the mode list above): an M
         // block is one staged row (pitch tw + 2 <= 128)
         if (a.npad != 16 && a.npad != 32) return Geometry{};
@@ -979,7 +1054,7 @@ Geometry plan(const ConvArgs& a, const TileCfg& t) {
         g.tiles = g.tiles_x * g.tiles_y * a.nb;
         return g;
     }
-    if (mode == 4) {
+    if (a.mode == 4) {
         // same grid, 16 output channels, column taps in N (see the mode list above)
         if (a.npad != 16) return Geometry{};
         const int H = a.hout, W = a.wout;
@@ -1026,7 +1101,9 @@ Geometry plan(const ConvArgs& a, const TileCfg& t) {
         g.tiles = g.tiles_x * g.tiles_y * a.nb;
         return g;
     }
-    // the grid the tile lives on: output grid for modes 0 and 1, coarse input grid for 2 and 3
+    // the grid the tile lives on: output grid for modes 0, 1 and 5, coarse input grid for 2 and 3
+    const bool rowsum = a.mode == 5;
+    const int mode = rowsum ? 0 : a.mode;
     const int H = mode >= 2 ? a.hin : a.hout, W = mode >= 2 ? a.win : a.wout;
     g.groups = (a.c0 + a.c1) / 16;
     g.groups0 = a.c0 / 16;
@@ -1053,16 +1130,16 @@ Geometry plan(const ConvArgs& a, const TileCfg& t) {
     // one buffer of up to 512 columns: twice the M blocks per stage (the weights of a
     // stage serve more pixels), but the MMAs of a tile wait for the previous epilogue
     g.nbuf = t.single ? 1 : 2;
-    if (t.single) acc_max = 512;
+    if (t.single) acc_max = rowsum ? 256 : 512;   // (mode 5: one MMA clears the buffer)
     const int maxmb = acc_max / (g.nph * a.npad);
     auto fill = [&](int rows) {
         g.rows = rows;
-        g.mb = (rows * g.pw + 127) / 128;
+        g.mb = rowsum ? rows : (rows * g.pw + 127) / 128;
         g.plane = ((rows + halo) * g.pw + SLACK_PX) * 16;
         g.pstride = (2 * g.plane + 127) / 128 * 128;
         g.stage = g.nplanes * g.pstride + g.wbytes;
     };
-    int rmax = (maxmb * 128) / g.pw;
+    int rmax = rowsum ? maxmb : (maxmb * 128) / g.pw;
     const int cap = t.rows_cap;
     if (cap > 0 && rmax > cap) rmax = cap;
     if (rmax > H) rmax = H;
@@ -1085,11 +1162,33 @@ Geometry plan(const ConvArgs& a, const TileCfg& t) {
     const int staged_px = mode == 1 ? (g.rows + 1) * g.pw : (g.rows + 2) * g.pw;
     g.tx = (uint32_t)(2 * g.nplanes * staged_px * 16 + g.wbytes);
     g.acc_cols = (uint32_t)(g.nph * g.mb * a.npad);
+    g.nzero = rowsum ? g.mb * a.npad : 0;
     uint32_t cols = 32;
     while (cols < (uint32_t)g.nbuf * g.acc_cols) cols <<= 1;
     g.tmem_cols = cols;
     g.tiles = g.tiles_x * g.tiles_y * a.nb * (g.psplit ? 2 : 1);
     return g;
+}
+
+// Cycles that an M = 128, K = 16 MMA holds the tensor core: its product, or the shared-memory reads of
+// its operands at 128 bytes per cycle (4 KB of A, 32 bytes of B per column).
+int mma_cycles(int n) { return std::max(n / 2, 32 + n / 4); }
+
+// Whether mode 5 (plan g5) takes fewer MMA cycles per output node and group than mode 0 (plan g0).  Mode
+// 5 reads A a third as often, but gives the lanes beyond a row's tile away (mode 0 packs rows), and its
+// tile ends carry fewer columns: 16 and 32 channels gain on every width that fills most of 128 lanes,
+// 64 channels have little to gain (their products already cost what A's reads do).
+bool rowsum_pays(const ConvArgs& a, const Geometry& g0, const Geometry& g5) {
+    if (g5.tiles <= 0 || 3 * a.npad > 256 || (size_t)g5.ns * g5.stage + ZERO_BYTES > 200 * 1024) return false;
+    if (g0.tiles <= 0) return false;
+    const double c0 = 9.0 * g0.mb * mma_cycles(a.npad) * g0.tiles;
+    double c5 = mma_cycles(g5.nzero) / (double)g5.groups;
+    for (int b = 0; b < g5.rows + 2; ++b) {
+        const int nt = (b < 2 ? b : 2) - (b < g5.rows ? 0 : b - g5.rows + 1) + 1;
+        c5 += 3.0 * mma_cycles(nt * a.npad);
+    }
+    c5 *= g5.tiles;
+    return c5 < 0.9 * c0;
 }
 
 int smem_per_sm() {
@@ -1198,7 +1297,15 @@ int plan_launch(const ConvArgs& a, const TileCfg& t, bool no_mode4, int* mode_ou
         g = plan(b, t);
         if (g.tiles <= 0 || (size_t)g.ns * g.stage > 200 * 1024) b.mode = 0;
     }
-    if (b.mode != 4 && b.mode != 6) g = plan(b, t);
+    if (b.mode != 4 && b.mode != 6) {
+        g = plan(b, t);
+        if (a.mode == 0 && !t.plain && !no_mode4) {
+            b.mode = 5;
+            const Geometry g5 = plan(b, t);
+            if (rowsum_pays(a, g, g5)) g = g5;
+            else b.mode = 0;
+        }
+    }
     *g_out = g;
     *mode_out = b.mode;
     if (g.tiles <= 0) return HELM_EINVAL;
@@ -1224,7 +1331,7 @@ int launch_cfg(const ConvArgs& a_in, cudaStream_t st, const TileCfg& t) {
     if (plan_launch(a, t, false, &mode, &g) != HELM_OK) return HELM_EINVAL;
     alignas(64) CUtensorMap tmw;
     if ((mode == 4 && !encode_w5(&tmw, a.w, a.c0 + a.c1, a.npad)) ||
-        (mode == 6 && !encode_w6(&tmw, a.w, a.c0 + a.c1, a.npad))) {
+        ((mode == 5 || mode == 6) && !encode_w6(&tmw, a.w, a.c0 + a.c1, a.npad))) {
         // no weight map for the variant: the plain same-grid kernel
         if (plan_launch(a, t, true, &mode, &g) != HELM_OK) return HELM_EINVAL;
     }
@@ -1243,7 +1350,7 @@ int launch_cfg(const ConvArgs& a_in, cudaStream_t st, const TileCfg& t) {
     } else {
         tm1 = tm0;
     }
-    if (a.mode != 4 && a.mode != 6) {
+    if (a.mode < 4) {
         const void* wsrc = a.mode == 2 ? (const void*)a.wup : (const void*)a.w;
         const int ntap = a.mode == 2 ? 16 : 9;
         g.w4 = encode_w4(&tmw, wsrc, a.c0 + a.c1, a.npad, ntap, g.psplit ? 8 : ntap) ? 1 : 0;
@@ -1251,6 +1358,7 @@ int launch_cfg(const ConvArgs& a_in, cudaStream_t st, const TileCfg& t) {
     }
     switch (a.mode) {
         case 4: ++g_launch_narrow; return launch_mode<4>(tm0, tm1, tmw, a, g, st);
+        case 5: return launch_mode<5>(tm0, tm1, tmw, a, g, st);
         case 6: ++g_launch_rowtaps; return launch_mode<6>(tm0, tm1, tmw, a, g, st);
         case 0: return launch_mode<0>(tm0, tm1, tmw, a, g, st);
         case 1: return launch_mode<1>(tm0, tm1, tmw, a, g, st);
@@ -1285,12 +1393,20 @@ int tune_and_launch(const ConvArgs& a, cudaStream_t st, const std::string& key, 
         c.stage_kb = b[0];
         c.ring_kb = b[1];
         c.narrow = 0;
+        c.plain = 1;
         cands.push_back(c);
     }
     {
         TileCfg c = base;
         c.rows_cap = 4;
         c.narrow = 0;
+        c.plain = 1;
+        cands.push_back(c);
+    }
+    if (a.mode == 0) {
+        TileCfg c = base;
+        c.narrow = 0;
+        c.plain = 1;
         cands.push_back(c);
     }
     if (a.mode == 0 && a.npad == 16 && base.narrow != 1) {
@@ -1307,6 +1423,7 @@ int tune_and_launch(const ConvArgs& a, cudaStream_t st, const std::string& key, 
         TileCfg c = base;
         c.narrow = 0;
         c.single = 1;
+        c.plain = 1;
         cands.push_back(c);
     }
     if (a.mode == 2) {
@@ -1372,7 +1489,10 @@ int launch_conv3x3_tma(const ConvArgs& a, cudaStream_t st, int narrow) {
     t.single = g_single.load();
     t.upsplit = g_upsplit.load();
     // explicit tiling knobs take precedence over the tuned table
-    if (t.rows_cap || t.stage_kb || t.ring_kb || t.single || t.upsplit) return launch_cfg(a, st, t);
+    if (t.rows_cap || t.stage_kb || t.ring_kb || t.single || t.upsplit) {
+        t.plain = 1;
+        return launch_cfg(a, st, t);
+    }
     const std::string key = shape_key(a);
     bool tune = false;
     {
@@ -1442,12 +1562,13 @@ extern "C" long long cnn_conv_rowtaps_launches(void) { return helm::g_launch_row
 
 // Tile plan of the TMA kernel for a layer shape (host only, no GPU needed): out19 =
 // {tiles, tw, rows, pw, mb, nph, nplanes, plane, pstride, wbytes, stage, ns, tmem_cols,
-// nslot, slot_cols, mode, nwg, chunk, nbuf}; narrow = 3 asks for the single-buffer tiling.
+// nslot, slot_cols, mode, nwg, chunk, nbuf}; narrow = 3 asks for the single-buffer tiling, 6 for the
+// tiling that a default launch takes (mode 5 or 0).
 // For checking the plan's bounds on the CPU.
 extern "C" int cnn_conv_plan(int mode, int c0, int c1, int npad, int hin, int win, int nb, int stage_kb,
                              int ring_kb, int rows_cap, int narrow, int* out19) {
     if (!out19 || mode < 0 || mode > 3 || c0 < 16 || c0 % 16 || c1 < 0 || c1 % 16 || nb < 1 || hin < 1 ||
-        win < 1 || (npad != 16 && npad % 32) || npad > 128 || narrow < 0 || narrow > 5) {
+        win < 1 || (npad != 16 && npad % 32) || npad > 128 || narrow < 0 || narrow > 6) {
         helm::set_error("cnn_conv_plan: invalid layer shape");
         return HELM_EINVAL;
     }
@@ -1467,7 +1588,8 @@ extern "C" int cnn_conv_plan(int mode, int c0, int c1, int npad, int hin, int wi
     t.ring_kb = ring_kb;
     t.narrow = narrow >= 3 ? 0 : narrow;
     t.single = narrow == 3 || narrow == 5 ? 1 : 0;
-    t.upsplit = narrow >= 4 ? 1 : 0;
+    t.upsplit = narrow == 4 || narrow == 5 ? 1 : 0;
+    t.plain = narrow != 6;
     helm::Geometry g{};
     int used = mode;
     const int s = helm::plan_launch(a, t, false, &used, &g);
