@@ -44,7 +44,7 @@
 //    of zeros clears the tile's columns, since every other one adds to rows in progress.  Mode 0
 //    at 32 -> 16 channels spends 76 % of the cycles on operand reads; 1024 x 512, 32 images, one
 //    GB300, mode 0 and mode 5: 344 and 305 us for one layer of 16 channels;
-//    the 29 layers of a network pass took 7.41 ms and take 7.17.
+//    the 29 layers of a network pass took 7.41 ms and take 7.17 (6.93 with the epilogue below).
 //  6 (16 or 32 output channels, same grid as mode 0) the three tap rows in N: an M block is
 //    one staged row (pitch tw + 2 <= 128, lanes >= tw dropped) and per 16-channel group takes
 //    three MMAs, one per column shift dx, computing D[b][x][(dy, o)] for N = 3 npad.  Output
@@ -159,6 +159,23 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
     return true;
 }
 
+// What the epilogue reads of one pixel's 16-channel segment, loaded ahead of its use.
+struct Pre2 {
+    uint4 a, b;
+};
+
+// The two halves of a packed BF16 pair, exactly.
+__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// (x, y) += (bx, by), two FP32 additions in one instruction.
+__device__ __forceinline__ void add2(float& x, float& y, float bx, float by) {
+    asm("{ .reg .b64 p, q;\n mov.b64 p, {%0, %1};\n mov.b64 q, {%2, %3};\n add.rn.f32x2 p, p, q;\n"
+        " mov.b64 {%0, %1}, p; }"
+        : "+f"(x), "+f"(y)
+        : "f"(bx), "f"(by));
+}
+
 // Tap t = (dy + 1) * 3 + (dx + 1) of output parity (py, px): whether it
 // contributes, and its A operand as (plane, offset in pixels from the tile's
 // staged pixel q).
@@ -190,8 +207,8 @@ __device__ __forceinline__ bool tap_source(int t, int py, int px, int pw, int* p
     }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __grid_constant__ CUtensorMap tm_x0,
+template <int MODE, bool ACT>
+__global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const __grid_constant__ CUtensorMap tm_x0,
                                                          const __grid_constant__ CUtensorMap tm_x1,
                                                          const __grid_constant__ CUtensorMap tm_w, ConvArgs a,
                                                          Geometry g) {
@@ -575,54 +592,63 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
         const long long hw_out = (long long)a.hout * a.wout;
         const size_t plane_out = (size_t)hw_out * 8;   // elements between 8-channel planes
         const int nblk = g.nph * g.mb;
-        const int step_y = 256 / g.pw, step_x = 256 - step_y * g.pw;
-        // one 16-channel segment of this thread's pixel: bias, residual, ReLU, store
-        auto segment = [&](float* vv, int n0, size_t ob, long long p) {
+        // The epilogue's instructions bound the layers of 16 channels: some 260 per 32 pixels when each
+        // value was rounded and packed by itself.  Pairs now: two additions, one conversion, one ReLU an
+        // instruction.  1024 x 512, 32 images, one GB300, 29 layers of a network pass: 7.17 -> 6.93 ms.
+        //
+        // The operand that the epilogue reads besides the accumulators: the residual, or the activation
+        // whose mask is applied.  It is loaded before the accumulators are waited for.
+        const __nv_bfloat16* pre_src = ACT || a.res ? a.res : a.gmask;
+        auto preload = [&](size_t ob, int n0, bool valid) {
+            Pre2 r{make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+            if (pre_src && valid) {
+                const __nv_bfloat16* q = pre_src + ob + (size_t)(n0 >> 3) * plane_out;
+                r.a = __ldg(reinterpret_cast<const uint4*>(q));
+                r.b = __ldg(reinterpret_cast<const uint4*>(q + plane_out));
+            }
+            return r;
+        };
+        // one 16-channel segment of pixel p = (image, pixel of it): bias, residual, ReLU, store
+        auto segment = [&](float* vv, int n0, size_t ob, long long p, const Pre2& pre) {
 #pragma unroll
             for (int i = 0; i < 16; i += 4) {
                 const float4 bb = *reinterpret_cast<const float4*>(bias_s + n0 + i);
-                vv[i] += bb.x;
-                vv[i + 1] += bb.y;
-                vv[i + 2] += bb.z;
-                vv[i + 3] += bb.w;
+                add2(vv[i], vv[i + 1], bb.x, bb.y);
+                add2(vv[i + 2], vv[i + 3], bb.z, bb.w);
             }
             const size_t o0 = ob + (size_t)(n0 >> 3) * plane_out;   // planes n0/8 and n0/8 + 1
+            const uint32_t pw8[8] = {pre.a.x, pre.a.y, pre.a.z, pre.a.w, pre.b.x, pre.b.y, pre.b.z, pre.b.w};
             if (a.res) {
-                uint4 r0 = __ldg(reinterpret_cast<const uint4*>(a.res + o0));
-                uint4 r1 = __ldg(reinterpret_cast<const uint4*>(a.res + o0 + plane_out));
-                const __nv_bfloat16* rb0 = reinterpret_cast<const __nv_bfloat16*>(&r0);
-                const __nv_bfloat16* rb1 = reinterpret_cast<const __nv_bfloat16*>(&r1);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    vv[i] += __bfloat162float(rb0[i]);
-                    vv[8 + i] += __bfloat162float(rb1[i]);
-                }
+                for (int i = 0; i < 8; ++i) add2(vv[2 * i], vv[2 * i + 1], bf_lo(pw8[i]), bf_hi(pw8[i]));
             }
-            if (a.relu) {
+            const bool packed = ACT || (!a.gmask && !a.out_fp32);
+            if (a.relu && !packed) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) vv[i] = fmaxf(vv[i], 0.0f);
             }
-            if (a.gmask) {
+            if (!ACT && a.gmask) {
                 // the gradient of an activation: what is there already, the ReLU mask, the skip's FP32 copy
                 if (a.gprior) {
                     const float4* q4 = reinterpret_cast<const float4*>(a.gprior + (size_t)p * a.npad + n0);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const float4 t = __ldg(q4 + q);
-                        vv[4 * q] += t.x;
-                        vv[4 * q + 1] += t.y;
-                        vv[4 * q + 2] += t.z;
-                        vv[4 * q + 3] += t.w;
+                        add2(vv[4 * q], vv[4 * q + 1], t.x, t.y);
+                        add2(vv[4 * q + 2], vv[4 * q + 3], t.z, t.w);
                     }
                 }
-                const uint4 m0 = __ldg(reinterpret_cast<const uint4*>(a.gmask + o0));
-                const uint4 m1 = __ldg(reinterpret_cast<const uint4*>(a.gmask + o0 + plane_out));
-                const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
-                const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
+                uint32_t mw[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) mw[i] = pw8[i];
+                if (a.res) {
+                    *reinterpret_cast<uint4*>(mw) = __ldg(reinterpret_cast<const uint4*>(a.gmask + o0));
+                    *reinterpret_cast<uint4*>(mw + 4) = __ldg(reinterpret_cast<const uint4*>(a.gmask + o0 + plane_out));
+                }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    if (!(__bfloat162float(mb0[i]) > 0.0f)) vv[i] = 0.0f;
-                    if (!(__bfloat162float(mb1[i]) > 0.0f)) vv[8 + i] = 0.0f;
+                    if (!(bf_lo(mw[i]) > 0.0f)) vv[2 * i] = 0.0f;
+                    if (!(bf_hi(mw[i]) > 0.0f)) vv[2 * i + 1] = 0.0f;
                 }
                 if (a.gres) {
                     float4* r4 = reinterpret_cast<float4*>(a.gres + (size_t)p * a.npad + n0);
@@ -637,7 +663,7 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                     }
                 }
             }
-            if (a.out_fp32) {
+            if (!ACT && a.out_fp32) {
                 float* yo = reinterpret_cast<float*>(a.y) + (size_t)p * a.cstore;
                 if ((a.cstore & 15) == 0) {
                     // whole 16-channel segments, 64-byte aligned: four 16-byte accesses
@@ -652,24 +678,26 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                         y4[q] = t;
                     }
                 } else if (a.accum) {
+#pragma unroll
                     for (int i = 0; i < 16; ++i)
                         if (n0 + i < a.cstore) yo[n0 + i] += vv[i];
                 } else {
+#pragma unroll
                     for (int i = 0; i < 16; ++i)
                         if (n0 + i < a.cstore) yo[n0 + i] = vv[i];
                 }
             } else {
-                uint4 w0, w1;
-                __nv_bfloat16* ob0 = reinterpret_cast<__nv_bfloat16*>(&w0);
-                __nv_bfloat16* ob1 = reinterpret_cast<__nv_bfloat16*>(&w1);
+                uint32_t w[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    ob0[i] = __float2bfloat16_rn(vv[i]);
-                    ob1[i] = __float2bfloat16_rn(vv[8 + i]);
+                    __nv_bfloat162 h = __floats2bfloat162_rn(vv[2 * i], vv[2 * i + 1]);
+                    // (rounding keeps the sign, so that ReLU may follow it)
+                    if (a.relu && packed) h = __hmax2(h, __nv_bfloat162(__nv_bfloat16_raw{0}, __nv_bfloat16_raw{0}));
+                    w[i] = *reinterpret_cast<const uint32_t*>(&h);
                 }
                 __nv_bfloat16* yq = reinterpret_cast<__nv_bfloat16*>(a.y) + o0;
-                *reinterpret_cast<uint4*>(yq) = w0;
-                *reinterpret_cast<uint4*>(yq + plane_out) = w1;
+                *reinterpret_cast<uint4*>(yq) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(yq + plane_out) = make_uint4(w[4], w[5], w[6], w[7]);
             }
         };
         if constexpr (MODE == 6) {
@@ -730,7 +758,7 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                         }
 #pragma unroll
                         for (int i = 0; i < 16; ++i) v0[i] += v1[i] + v2[i];
-                        if (valid) segment(v0, c0, ob, p);
+                        if (valid) segment(v0, c0, ob, p, preload(ob, c0, true));
                     }
                 }
                 jslot += g.mb;
@@ -778,62 +806,67 @@ __global__ void __launch_bounds__(threads_of(MODE)) conv3x3_tma_kernel(const __g
                     for (int c = 0; c < 16; ++c)
                         v[c] = d[c] + __shfl_down_sync(0xffffffffu, d[16 + c], 1) +
                                __shfl_down_sync(0xffffffffu, d[32 + c], 2);
-                    if (valid) segment(v, 0, ob, p);
+                    if (valid) segment(v, 0, ob, p, preload(ob, 0, true));
                 }
             }
         } else {
             for (int k = 0; k < ntiles; ++k) {
                 const int acc = g.nbuf == 2 ? (k & 1) : 0;
                 const uint32_t par = (uint32_t)((g.nbuf == 2 ? (k >> 1) : k) & 1);
-                if (!wait_bar(&tfull[acc], par, abort_v, 128)) { *abort_v = 1; break; }
-                tc::tc_fence_after_sync();
                 int b, xs, ys;
                 tile_coords(k, b, xs, ys);
                 const uint32_t dbase = lane_base + (uint32_t)acc * g.acc_cols;
                 const size_t img_base = (size_t)b * (size_t)(a.npad >> 3) * (size_t)hw_out * 8;
-                int m_prev = -4, yy = 0, xx = 0;
-                for (int bi = wg; bi < nblk; bi += 2) {
+                // output pixel of this thread's row of block bi (-1: none)
+                auto pixel = [&](int bi) {
+                    if (bi >= nblk) return -1;
                     const int ph = MODE == 5 ? 0 : bi / g.mb, m = bi - ph * g.mb;
-                    if (MODE == 5) {
-                        yy = bi;      // a block is an output row
-                        xx = row;
-                    } else if (m != m_prev + 2) {
+                    int yy = m, xx = row;        // mode 5: a block is an output row
+                    if (MODE != 5) {
                         const int q = m * 128 + row;
                         yy = q / g.pw;
                         xx = q - yy * g.pw;
-                    } else {
-                        // the warpgroup's next block of the same phase lies 256 pixels further on
-                        yy += step_y;
-                        xx += step_x;
-                        if (xx >= g.pw) {
-                            xx -= g.pw;
-                            ++yy;
-                        }
                     }
-                    m_prev = m;
                     int oy = ys + yy, ox = xs + xx;
                     if (MODE == 2 || MODE == 3) {
                         oy = 2 * oy + (g.psplit ? tile_py(k) : ph >> 1);
                         ox = 2 * ox + (g.psplit ? ph : ph & 1);
                     }
-                    const bool valid = xx < g.tw && yy < g.rows && oy < a.hout && ox < a.wout;
-                    const long long pix = (long long)oy * a.wout + ox;
-                    const size_t ob = img_base + (size_t)pix * 8;   // channel 0 of this pixel
+                    return xx < g.tw && yy < g.rows && oy < a.hout && ox < a.wout ? oy * a.wout + ox : -1;
+                };
+                // (16 channels: the next block's operand is under way while this one is finished)
+                int pix = pixel(wg);
+                Pre2 pre{};
+                if (ACT && a.npad == 16) pre = preload(img_base + (size_t)(unsigned)pix * 8, 0, pix >= 0);
+                if (!wait_bar(&tfull[acc], par, abort_v, 128)) { *abort_v = 1; break; }
+                tc::tc_fence_after_sync();
+                for (int bi = wg; bi < nblk; bi += 2) {
+                    const int next = pixel(bi + 2);
+                    const size_t ob = img_base + (size_t)(unsigned)pix * 8;   // channel 0 of this pixel
                     const long long p = (long long)b * hw_out + pix;
                     const uint32_t tcol = dbase + (uint32_t)((MODE == 5 ? g.rows - 1 - bi : bi) * a.npad);
                     if (a.npad == 16) {
+                        Pre2 pn{};
+                        if (ACT) pn = preload(img_base + (size_t)(unsigned)next * 8, 0, next >= 0);
+                        else pre = preload(ob, 0, pix >= 0);
                         float v[16];
                         tc::tmem_ld16(tcol, v);
-                        if (valid) segment(v, 0, ob, p);
+                        if (pix >= 0) segment(v, 0, ob, p, pre);
+                        if (ACT) pre = pn;
                     } else {
                         for (int c0 = 0; c0 < a.npad; c0 += 32) {
+                            const Pre2 p0 = preload(ob, c0, pix >= 0);
+                            Pre2 p1{};
+                            if (ACT) p1 = preload(ob, c0 + 16, pix >= 0);
                             float v[32];
                             tc::tmem_ld32(tcol + (uint32_t)c0, v);
-                            if (!valid) continue;
-                            segment(v, c0, ob, p);
-                            segment(v + 16, c0 + 16, ob, p);
+                            if (pix < 0) continue;
+                            segment(v, c0, ob, p, p0);
+                            if (!ACT) p1 = preload(ob, c0 + 16, true);
+                            segment(v + 16, c0 + 16, ob, p, p1);
                         }
                     }
+                    pix = next;
                 }
                 // this thread's TMEM reads of the buffer are complete (tcgen05.ld waited)
                 tc::tc_fence_before_sync();
@@ -1217,14 +1250,14 @@ int sm_count() {
     return n > 0 ? n : 148;
 }
 
-template <int MODE>
-int launch_mode(const CUtensorMap& tm0, const CUtensorMap& tm1, const CUtensorMap& tmw, const ConvArgs& a,
+template <int MODE, bool ACT>
+int launch_kernel(const CUtensorMap& tm0, const CUtensorMap& tm1, const CUtensorMap& tmw, const ConvArgs& a,
                 const Geometry& g, cudaStream_t st) {
     static std::once_flag once;
     std::call_once(once, [] {
-        cudaFuncSetAttribute(conv3x3_tma_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(conv3x3_tma_kernel<MODE, ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         // all of the unified L1/shared storage as shared memory: two CTAs of ~100 KB per SM
-        cudaFuncSetAttribute(conv3x3_tma_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        cudaFuncSetAttribute(conv3x3_tma_kernel<MODE, ACT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     });
     const size_t smem = (size_t)g.ns * g.stage;
     // two CTAs per SM when two fit the 512 TMEM columns, else one; a shared-memory
@@ -1237,7 +1270,7 @@ int launch_mode(const CUtensorMap& tm0, const CUtensorMap& tm1, const CUtensorMa
     static std::once_flag attrs;
     std::call_once(attrs, [] {
         cudaFuncAttributes fa;
-        if (cudaFuncGetAttributes(&fa, conv3x3_tma_kernel<MODE>) == cudaSuccess) {
+        if (cudaFuncGetAttributes(&fa, conv3x3_tma_kernel<MODE, ACT>) == cudaSuccess) {
             regs = fa.numRegs;
             static_smem = (int)fa.sharedSizeBytes;
         } else {
@@ -1257,8 +1290,18 @@ int launch_mode(const CUtensorMap& tm0, const CUtensorMap& tm1, const CUtensorMa
     g_last_launch[3] = (int)smem_req;
     g_last_launch[4] = regs;
     g_last_launch[5] = static_smem;
-    { conv3x3_tma_kernel<MODE><<<(unsigned)grid, NT, smem_req, st>>>(tm0, tm1, tmw, a, g); count_launch(); }
+    { conv3x3_tma_kernel<MODE, ACT><<<(unsigned)grid, NT, smem_req, st>>>(tm0, tm1, tmw, a, g); count_launch(); }
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_ECUDA;
+}
+
+// ACT: the instance for BF16 activations alone (no gradient output, no FP32 output), which holds no
+// registers for the rest: two CTAs per SM with a block's operand loaded ahead.
+template <int MODE>
+int launch_mode(const CUtensorMap& tm0, const CUtensorMap& tm1, const CUtensorMap& tmw, const ConvArgs& a,
+                const Geometry& g, cudaStream_t st) {
+    if constexpr (MODE != 4 && MODE != 6)
+        if (!a.gmask && !a.out_fp32) return launch_kernel<MODE, true>(tm0, tm1, tmw, a, g, st);
+    return launch_kernel<MODE, false>(tm0, tm1, tmw, a, g, st);
 }
 
 }  // namespace
