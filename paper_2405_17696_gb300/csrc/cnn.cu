@@ -97,20 +97,23 @@ int malloc_m(cnn_model* m, T** p, size_t n) {
     return HELM_OK;
 }
 
-// master FP32 [cout][9][cin] + bias -> padded BF16 [npad][9][cin_pad] + FP32 bias [npad]
+// master FP32 [cout][9][cin] + bias -> padded BF16 [npad][9][cin_pad], the same in staged order, FP32 bias [npad]
 __global__ void pack_weights_kernel(const float* __restrict__ master, long long off, int cin, int cout, int cin_pad,
-                                    int npad, __nv_bfloat16* __restrict__ w, float* __restrict__ b) {
+                                    int npad, __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wst,
+                                    float* __restrict__ b) {
     const int total = npad * 9 * cin_pad;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         int ci = i % cin_pad, t = (i / cin_pad) % 9, co = i / (9 * cin_pad);
         float v = (co < cout && ci < cin) ? master[off + ((long long)co * 9 + t) * cin + ci] : 0.0f;
-        w[i] = __float2bfloat16_rn(v);
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        w[i] = h;
+        wst[staged_weight(co, t, ci, npad)] = h;
         if (i < npad) b[i] = i < cout ? master[off + (long long)cout * 9 * cin + i] : 0.0f;
     }
 }
 
-// master FP32 [cout][9][cin] -> the phase-merged BF16 weights [npad][16][cin_pad] of an up
-// layer: row up_merged_index(py, px, dy, dx) holds the sum, in FP32, of the taps (dy, dx) of
+// master FP32 [cout][9][cin] -> the phase-merged BF16 weights of an up layer, in staged
+// order: row up_merged_index(py, px, dy, dx) holds the sum, in FP32, of the taps (dy, dx) of
 // output parity (py, px) that read the same coarse node, rounded once
 __global__ void pack_up_weights_kernel(const float* __restrict__ master, long long off, int cin, int cout,
                                        int cin_pad, int npad, __nv_bfloat16* __restrict__ wup) {
@@ -123,7 +126,7 @@ __global__ void pack_up_weights_kernel(const float* __restrict__ master, long lo
             for (int t = 0; t < 9; ++t)
                 if (up_merged_index(ph >> 1, ph & 1, t / 3 - 1, t % 3 - 1) == r)
                     v += master[off + ((long long)co * 9 + t) * cin + ci];
-        wup[i] = __float2bfloat16_rn(v);
+        wup[staged_up_weight(co, r, ci, npad)] = __float2bfloat16_rn(v);
     }
 }
 
@@ -397,7 +400,7 @@ __global__ void solver_output_kernel(const float* __restrict__ out, const float*
 // Rebuild the padded BF16 weights from the FP32 master parameters.
 int cnn_refresh_weights(cnn_model* m, cudaStream_t st) {
     for (const Layer& l : m->layers) {
-        { pack_weights_kernel<<<64, 256, 0, st>>>(m->master, l.off, l.cin, l.cout, l.cin_pad, l.npad, l.w, l.b); count_launch(); }
+        { pack_weights_kernel<<<64, 256, 0, st>>>(m->master, l.off, l.cin, l.cout, l.cin_pad, l.npad, l.w, l.wst, l.b); count_launch(); }
         if (l.wup) { pack_up_weights_kernel<<<64, 256, 0, st>>>(m->master, l.off, l.cin, l.cout, l.cin_pad, l.npad, l.wup); count_launch(); }
         HELM_CK(cudaGetLastError());
     }
@@ -712,6 +715,7 @@ int create_zero(cnn_model** out, int levels, const int* widths) {
     for (Layer& l : m->layers) {
         if (s) break;
         s = malloc_m(m, &l.w, (size_t)l.npad * 9 * l.cin_pad);
+        if (!s) s = malloc_m(m, &l.wst, (size_t)l.npad * 9 * l.cin_pad);
         if (!s && l.mode == 2) s = malloc_m(m, &l.wup, (size_t)l.npad * 16 * l.cin_pad);
         if (!s) s = malloc_m(m, &l.b, (size_t)l.npad);
     }
@@ -720,6 +724,7 @@ int create_zero(cnn_model** out, int levels, const int* widths) {
     cudaMemset(m->err, 0, sizeof(int));
     for (Layer& l : m->layers) {
         cudaMemset(l.w, 0, (size_t)l.npad * 9 * l.cin_pad * sizeof(__nv_bfloat16));
+        cudaMemset(l.wst, 0, (size_t)l.npad * 9 * l.cin_pad * sizeof(__nv_bfloat16));
         if (l.wup) cudaMemset(l.wup, 0, (size_t)l.npad * 16 * l.cin_pad * sizeof(__nv_bfloat16));
         cudaMemset(l.b, 0, (size_t)l.npad * sizeof(float));
     }
@@ -863,7 +868,7 @@ int cnn_conv3x3(const float* x0, int c0, const float* x1, int c1, int x1_bcast, 
     const long long nin = (long long)nb * hin * win, nin1 = (long long)(x1_bcast ? 1 : nb) * hin * win;
     const long long nout = (long long)nb * hout * wout;
     float *fx0 = nullptr, *fx1 = nullptr, *fw = nullptr, *fb = nullptr, *fr = nullptr, *fy = nullptr, *bp = nullptr;
-    __nv_bfloat16 *bx0 = nullptr, *bx1 = nullptr, *bw = nullptr, *bwup = nullptr, *br = nullptr, *by = nullptr;
+    __nv_bfloat16 *bx0 = nullptr, *bx1 = nullptr, *bw = nullptr, *bwst = nullptr, *bwup = nullptr, *br = nullptr, *by = nullptr;
     int* err = nullptr;
     int s = HELM_OK;
     auto ck = [&](cudaError_t e) { if (e != cudaSuccess && s == HELM_OK) { set_error(cudaGetErrorString(e)); s = HELM_ECUDA; } };
@@ -872,6 +877,7 @@ int cnn_conv3x3(const float* x0, int c0, const float* x1, int c1, int x1_bcast, 
     if (c1) { ck(cudaMalloc(&fx1, nin1 * c1 * sizeof(float))); ck(cudaMalloc(&bx1, nin1 * cp1 * sizeof(__nv_bfloat16))); }
     ck(cudaMalloc(&fw, (size_t)cout * 9 * cin * sizeof(float) + cout * sizeof(float)));
     ck(cudaMalloc(&bw, (size_t)npad * 9 * cinp * sizeof(__nv_bfloat16)));
+    ck(cudaMalloc(&bwst, (size_t)npad * 9 * cinp * sizeof(__nv_bfloat16)));
     if (mode == 2) ck(cudaMalloc(&bwup, (size_t)npad * 16 * cinp * sizeof(__nv_bfloat16)));
     ck(cudaMalloc(&bp, npad * sizeof(float)));
     ck(cudaMalloc(&fy, nout * cout * sizeof(float)));
@@ -895,16 +901,19 @@ int cnn_conv3x3(const float* x0, int c0, const float* x1, int c1, int x1_bcast, 
         std::vector<float> hw((size_t)cout * 9 * cin + cout);
         ck(cudaMemcpy(hw.data(), fw, hw.size() * sizeof(float), cudaMemcpyDeviceToHost));
         std::vector<__nv_bfloat16> hbw((size_t)npad * 9 * cinp, __float2bfloat16_rn(0.0f));
+        std::vector<__nv_bfloat16> hst(hbw.size(), __float2bfloat16_rn(0.0f));
         std::vector<float> hb(npad, 0.0f);
         for (int co = 0; co < cout; ++co) {
             for (int t = 0; t < 9; ++t)
                 for (int ci = 0; ci < cin; ++ci) {
                     int cpi = ci < c0 ? ci : cp0 + (ci - c0);
                     hbw[((size_t)co * 9 + t) * cinp + cpi] = __float2bfloat16_rn(hw[((size_t)co * 9 + t) * cin + ci]);
+                    hst[staged_weight(co, t, cpi, npad)] = hbw[((size_t)co * 9 + t) * cinp + cpi];
                 }
             hb[co] = hw[(size_t)cout * 9 * cin + co];
         }
         ck(cudaMemcpy(bw, hbw.data(), hbw.size() * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice));
+        ck(cudaMemcpy(bwst, hst.data(), hst.size() * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice));
         if (mode == 2) {
             // the phase-merged weights of the up layer (summed in FP32 in tap order, rounded once)
             std::vector<float> acc((size_t)npad * 16 * cinp, 0.0f);
@@ -919,7 +928,9 @@ int cnn_conv3x3(const float* x0, int c0, const float* x1, int c1, int x1_bcast, 
                         }
                     }
             std::vector<__nv_bfloat16> hup(acc.size());
-            for (size_t i = 0; i < acc.size(); ++i) hup[i] = __float2bfloat16_rn(acc[i]);
+            for (size_t i = 0; i < acc.size(); ++i)
+                hup[staged_up_weight((int)(i / (16 * cinp)), (int)(i / cinp % 16), (int)(i % cinp), npad)] =
+                    __float2bfloat16_rn(acc[i]);
             ck(cudaMemcpy(bwup, hup.data(), hup.size() * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice));
         }
         ck(cudaMemcpy(bp, hb.data(), hb.size() * sizeof(float), cudaMemcpyHostToDevice));
@@ -929,7 +940,7 @@ int cnn_conv3x3(const float* x0, int c0, const float* x1, int c1, int x1_bcast, 
         ConvArgs a;
         a.x0 = bx0; a.c0 = cp0; a.x1 = bx1; a.c1 = cp1; a.x1_bcast = x1_bcast; a.x1_map = nullptr;
         a.nb = nb; a.hin = hin; a.win = win; a.hout = hout; a.wout = wout; a.mode = mode;
-        a.w = bw; a.wup = bwup; a.bias = bp; a.res = br; a.y = by; a.npad = npad; a.cstore = cout; a.relu = relu;
+        a.w = bw; a.wst = bwst; a.wup = bwup; a.bias = bp; a.res = br; a.y = by; a.npad = npad; a.cstore = cout; a.relu = relu;
         a.out_fp32 = 0;
         a.accum = 0;
         a.err = err;
@@ -948,7 +959,7 @@ int cnn_conv3x3(const float* x0, int c0, const float* x1, int c1, int x1_bcast, 
         if (!s) ck(cudaMemcpy(y, fy, nout * cout * sizeof(float), cudaMemcpyDefault));
     }
     cudaFree(fx0); cudaFree(fx1); cudaFree(fw); cudaFree(fb); cudaFree(fr); cudaFree(fy); cudaFree(bp);
-    cudaFree(bx0); cudaFree(bx1); cudaFree(bw); cudaFree(bwup); cudaFree(br); cudaFree(by); cudaFree(err);
+    cudaFree(bx0); cudaFree(bx1); cudaFree(bw); cudaFree(bwst); cudaFree(bwup); cudaFree(br); cudaFree(by); cudaFree(err);
     return s;
 }
 
@@ -1032,7 +1043,7 @@ int cnn_conv3x3_backward(const float* x0, int c0, const float* x1, int c1, int x
         const int c = part ? c1 : c0, cp = part ? cp1 : cp0;
         if (!out || c == 0) continue;
         float* target = (float*)alloc(nin * cp * sizeof(float));
-        auto* Wt = (__nv_bfloat16*)alloc((size_t)cp * 9 * npad * sizeof(__nv_bfloat16));
+        auto* Wt = (__nv_bfloat16*)alloc((size_t)2 * cp * 9 * npad * sizeof(__nv_bfloat16));
         float* fine = mode == 2 ? (float*)alloc(nout * cp * sizeof(float)) : nullptr;
         if (s) break;
         GradOut go;

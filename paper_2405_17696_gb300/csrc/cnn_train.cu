@@ -105,13 +105,16 @@ __global__ void mask_to_bf16_vec_kernel(const float* __restrict__ G, const __nv_
     }
 }
 
-// Wt[ci][t][co] = W[co][flip ? 8 - t : t][off + ci]   (dgrad weights of one input part)
+// Wt[ci][t][co] = W[co][flip ? 8 - t : t][off + ci]   (dgrad weights of one input part), then the same
+// in staged order (staged_weight)
 __global__ void transpose_weights_kernel(const __nv_bfloat16* __restrict__ W, int npad, int cin_pad, int off,
                                          int cpart, int flip, __nv_bfloat16* __restrict__ Wt) {
     const int total = cpart * 9 * npad;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int co = i % npad, t = (i / npad) % 9, ci = i / (9 * npad);
-        Wt[i] = W[((size_t)co * 9 + (flip ? 8 - t : t)) * cin_pad + off + ci];
+        const __nv_bfloat16 h = W[((size_t)co * 9 + (flip ? 8 - t : t)) * cin_pad + off + ci];
+        Wt[i] = h;
+        Wt[(size_t)total + staged_weight(ci, t, co, cpart)] = h;
     }
 }
 
@@ -454,7 +457,7 @@ int layer_wgrad(const __nv_bfloat16* x0, int c0, const __nv_bfloat16* x1, int c1
 // The input gradient W^T g of one input part (channels off .. off + cp - 1 of the layer's padded input) on
 // the tensor cores, written as `out` says: 'same' -> same-grid convolution with transposed, tap-flipped
 // weights; 'down' -> the transpose-of-down mode; 'up' -> a same-grid convolution on the fine grid, then
-// a 2 x 2 sum.  Wt: scratch of cp x 9 x npad BF16; fine: scratch of nb x hout x wout x cp FP32 (mode 2).
+// a 2 x 2 sum.  Wt: scratch of 2 x cp x 9 x npad BF16; fine: scratch of nb x hout x wout x cp FP32 (mode 2).
 int layer_dgrad(const __nv_bfloat16* g, int npad, const __nv_bfloat16* W, int cin_pad, int off, int cp, int mode,
                 int nb, int hin, int win, int hout, int wout, const GradOut& out, __nv_bfloat16* Wt, float* fine,
                 int* err, cudaStream_t st, const helm_ctx* prof_ctx) {
@@ -464,7 +467,7 @@ int layer_dgrad(const __nv_bfloat16* g, int npad, const __nv_bfloat16* W, int ci
     }
     ConvArgs ca;
     ca.x0 = g; ca.c0 = npad; ca.x1 = nullptr; ca.c1 = 0; ca.x1_bcast = 0; ca.x1_map = nullptr;
-    ca.nb = nb; ca.w = Wt; ca.bias = nullptr; ca.res = nullptr; ca.npad = cp; ca.cstore = cp;
+    ca.nb = nb; ca.w = Wt; ca.wst = Wt + (size_t)cp * 9 * npad; ca.bias = nullptr; ca.res = nullptr; ca.npad = cp; ca.cstore = cp;
     ca.relu = 0; ca.out_fp32 = 1; ca.accum = 0; ca.err = err;
     ca.hin = hout; ca.win = wout;
     if (mode == 0 || mode == 1) {
@@ -630,7 +633,7 @@ class Backward {
                 if (pit == producer.end()) continue;
                 const int shared = part == 1 && op.x1_bcast != 0;
                 const long long nin = (long long)op.nb * op.hin * op.win;
-                __nv_bfloat16* Wt = (__nv_bfloat16*)alloc((size_t)cp * 9 * L.npad * sizeof(__nv_bfloat16));
+                __nv_bfloat16* Wt = (__nv_bfloat16*)alloc((size_t)2 * cp * 9 * L.npad * sizeof(__nv_bfloat16));
                 float* fine = L.mode == 2 ? (float*)alloc((size_t)nout * cp * sizeof(float)) : nullptr;
                 if (!ok_) break;
                 auto dgrad = [&](const GradOut& o) {

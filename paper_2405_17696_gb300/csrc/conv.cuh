@@ -27,6 +27,19 @@ __host__ __device__ __forceinline__ int up_merged_index(int py, int px, int dy, 
     return (2 * py + px) * 4 + 2 * up_phase_tap(py, dy) + up_phase_tap(px, dx);
 }
 
+// The weights in the order in which the tensor-map kernel stages a group of 16 input channels: [group]
+// [dx][half][dy][npad][8 channels], and an up layer's merged taps r as [group][r][half][npad][8], so that
+// a group is one contiguous copy.  (A tensor-map box of the plain layout has 16-byte rows, 18 npad of
+// them per stage.  1024 x 512, 32 images, one GB300, 29 layers of a network pass: 6.93 -> 5.04 ms.)
+__host__ __device__ __forceinline__ size_t staged_weight(int co, int t, int ci, int npad) {
+    const int g = ci >> 4, half = (ci >> 3) & 1;
+    return (((((size_t)g * 3 + t % 3) * 2 + half) * 3 + t / 3) * npad + co) * 8 + (ci & 7);
+}
+__host__ __device__ __forceinline__ size_t staged_up_weight(int co, int r, int ci, int npad) {
+    const int g = ci >> 4, half = (ci >> 3) & 1;
+    return ((((size_t)g * 16 + r) * 2 + half) * npad + co) * 8 + (ci & 7);
+}
+
 struct ConvArgs {
     const __nv_bfloat16* x0;   // [nb][c0/8][hin][win][8] (chunked layout, see nc8)
     int c0;
@@ -40,8 +53,10 @@ struct ConvArgs {
                                // 3 transpose of down: output on the fine grid, tap d of output node f reads
                                //   input node (f - 1 - d) / 2 when that is an integer inside the input
     const __nv_bfloat16* w;    // [npad][9][c0 + c1]
-    const __nv_bfloat16* wup = nullptr;   // mode 2: the phase-merged weights [npad][16][c0 + c1]
-                                          // (up_merged_index), which the tensor-map kernel needs
+    // what the tensor-map kernel reads instead: the same weights in staged order (staged_weight), and for
+    // mode 2 the phase-merged ones (up_merged_index, staged_up_weight)
+    const __nv_bfloat16* wst = nullptr;
+    const __nv_bfloat16* wup = nullptr;
     const float* bias;         // [npad], or nullptr: none
     const __nv_bfloat16* res;  // [nb][npad/8][hout][wout][8] added before the activation, or nullptr
     void* y;                   // bf16 [nb][npad/8][hout][wout][8], or fp32 [nb][hout][wout][cstore]

@@ -9,7 +9,7 @@
 // block of 128 output pixels is then a plane seen from a start address shifted
 // by the tap's offset in pixels; no gather.  Pixels outside the image are
 // zero-filled by TMA.  The weights of the group (9 taps x 16 channels x N)
-// arrive by TMA in the same layout.
+// arrive in the same layout, by one contiguous copy (staged_weight).
 //
 // Sampling modes (output node -> input nodes of its taps):
 //  0 same grid   (y, x)           -> (y + dy, x + dx); one (rows+2) x (tw+2) halo plane per 8 channels.
@@ -44,7 +44,8 @@
 //    of zeros clears the tile's columns, since every other one adds to rows in progress.  Mode 0
 //    at 32 -> 16 channels spends 76 % of the cycles on operand reads; 1024 x 512, 32 images, one
 //    GB300, mode 0 and mode 5: 344 and 305 us for one layer of 16 channels;
-//    the 29 layers of a network pass took 7.41 ms and take 7.17 (6.93 with the epilogue below).
+//    the 29 layers of a network pass took 7.41 ms and took 7.17 (5.04 with the epilogue below and
+//    the weights' contiguous copy).
 //  6 (16 or 32 output channels, same grid as mode 0) the three tap rows in N: an M block is
 //    one staged row (pitch tw + 2 <= 128, lanes >= tw dropped) and per 16-channel group takes
 //    three MMAs, one per column shift dx, computing D[b][x][(dy, o)] for N = 3 npad.  Output
@@ -126,7 +127,6 @@ struct Geometry {
     int pstride;             // bytes between parity sub-planes (two planes, rounded up to 128 B)
     int nplanes;             // parity sub-planes: 1, or 4 in mode 1
     int wbytes;              // bytes of one group's weights (9 taps x 2 chunks x npad rows x 16 B)
-    int w4;                  // weights by one 4-D TMA box (1) or 18 2-D boxes (0)
     int nslot, slot_cols;    // modes 4 and 6: TMEM slots (an M block / a staged row each) and their columns
     int nbuf;                // modes 0-3: TMEM accumulator buffers (2: the epilogue drains one while
                              // the MMAs fill the other; 1: twice the M blocks per tile)
@@ -253,7 +253,6 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
     tc::tc_fence_after_sync();
     const uint32_t tmem = tmem_base;
     volatile int* abort_v = &abort_flag;
-    const int cin = a.c0 + a.c1;
     const int G = g.groups;
     const int ntiles = g.tiles > (int)blockIdx.x ? (g.tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int chunk_bytes = g.plane;                 // K-adjacent core matrices (LBO)
@@ -274,7 +273,6 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
 
     if (tid == EPI) {
         // ---------------- TMA producer ----------------
-        const uint32_t wplane = (uint32_t)a.npad * 16;
         long long j = 0;
         int s = 0, wraps = 0;   // j % ns and j / ns as counters
         bool ok = true;
@@ -310,20 +308,18 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
                     }
                 }
                 unsigned char* ws = st + wofs;
-                if (MODE == 4 || MODE == 5 || MODE == 6) {
-                    // mode 4 [dy][half][dx][npad][8]: the B operand of tap row dy is 3 npad rows (dx, o);
-                    // modes 5 and 6 [dx][half][dy][npad][8]: the B operand of column shift dx is 3 npad rows (dy, o)
+                if (MODE == 4) {
+                    // [dy][half][dx][npad][8]: the B operand of tap row dy is 3 npad rows (dx, o)
                     tc::tma_load_5d(ws, &tm_w, 0, 0, 0, 2 * gi, 0, &full[s]);
-                } else if (g.w4) {
-                    // split parities: the 8 merged taps of the tile's row parity
-                    tc::tma_load_4d(ws, &tm_w, 0, 0, 2 * gi, 8 * tile_py(k), &full[s]);
+                } else if (MODE == 2) {
+                    // the merged taps of all parities, or of the tile's row parity
+                    const size_t gb = (size_t)512 * a.npad;   // bytes of a group: 16 taps x 16 channels
+                    tc::bulk_load(ws, reinterpret_cast<const unsigned char*>(a.wup) + gi * gb + tile_py(k) * (gb / 2),
+                                  (uint32_t)g.wbytes, &full[s]);
                 } else {
-                    const int t0 = 8 * tile_py(k);
-                    const int nt = MODE == 2 ? (g.psplit ? 8 : 16) : 9;
-                    for (int tap = 0; tap < nt; ++tap)
-                        for (int h = 0; h < 2; ++h)
-                            tc::tma_load_2d(ws + (tap * 2 + h) * wplane, &tm_w, (t0 + tap) * cin + gi * 16 + h * 8, 0,
-                                            &full[s]);
+                    // [dx][half][dy][npad][8]
+                    tc::bulk_load(ws, reinterpret_cast<const unsigned char*>(a.wst) + (size_t)gi * g.wbytes,
+                                  (uint32_t)g.wbytes, &full[s]);
                 }
             }
         }
@@ -346,10 +342,10 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
         const uint32_t wplane = (uint32_t)a.npad * 16;
         // descriptors with a zero start address: the start (bits 0-13, 16-byte units) is added per MMA
         const uint64_t adesc0 = tc::smem_desc(0u, (uint32_t)chunk_bytes, 128);
-        const uint64_t bdesc0 = tc::smem_desc(0u, wplane, 128);
+        // (K halves of B: a merged tap's are npad rows apart, the others' 3 npad, see staged_weight)
+        const uint64_t bdesc0 = tc::smem_desc(0u, MODE == 2 ? wplane : 3u * wplane, 128);
         const uint32_t a_lo0 = (uint32_t)adesc0, a_hi = (uint32_t)(adesc0 >> 32);
         const uint32_t b_lo0 = (uint32_t)bdesc0, b_hi = (uint32_t)(bdesc0 >> 32);
-        const uint32_t tap_b16 = (2u * wplane) >> 4;   // B planes of one tap, 16-byte units
         long long j = 0;
         bool ok = true;
         if constexpr (MODE == 4) {
@@ -549,7 +545,7 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
                             ao[tap] = a_lo0 + a16 + (uint32_t)(pl * (g.pstride >> 4) + off);
                         }
                         // B of the parity's first tap (mode 2: the merged weights are [parity][4 taps])
-                        const uint32_t bph = MODE == 2 ? bw_lo + (uint32_t)(ph * 4) * tap_b16 : bw_lo;
+                        const uint32_t bph = MODE == 2 ? bw_lo + (uint32_t)(ph * 8 * a.npad) : bw_lo;
                         uint32_t d = dbase + (uint32_t)(ph * g.mb * a.npad);
                         for (int m = 0; m < g.mb; ++m, d += (uint32_t)a.npad) {
                             const uint32_t mo = (uint32_t)(m * 128);   // 128 pixels of 16 bytes
@@ -559,7 +555,8 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
                                 if (!use[tap]) continue;
                                 if (leader) {
                                     const uint64_t ad = ((uint64_t)a_hi << 32) | (ao[tap] + mo);
-                                    const uint64_t bd = ((uint64_t)b_hi << 32) | (bph + (uint32_t)tap * tap_b16);
+                                    const uint64_t bd = ((uint64_t)b_hi << 32) |
+                                                        (bph + (uint32_t)((MODE == 2 ? 2 * tap : tap % 3 * 6 + tap / 3) * a.npad));
                                     tc::mma_bf16(d, ad, bd, idesc, accum);
                                 }
                                 accum = 1u;
@@ -594,7 +591,7 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
         const int nblk = g.nph * g.mb;
         // The epilogue's instructions bound the layers of 16 channels: some 260 per 32 pixels when each
         // value was rounded and packed by itself.  Pairs now: two additions, one conversion, one ReLU an
-        // instruction.  1024 x 512, 32 images, one GB300, 29 layers of a network pass: 7.17 -> 6.93 ms.
+        // instruction.  1024 x 512, 32 images, one GB300, 29 layers of a network pass: 7.17 -> 6.93 ms, before the weights' contiguous copy.
         //
         // The operand that the epilogue reads besides the accumulators: the residual, or the activation
         // whose mask is applied.  It is loaded before the accumulators are waited for.
@@ -954,22 +951,6 @@ bool tma_map_act(CUtensorMap* m, const void* base, int c, int w, int h, int n, i
 
 namespace {
 
-// weights [npad][ntap][cin] (ntap 9, or 16 merged taps in mode 2) viewed as a 4-D
-// tensor (8 channels, npad rows, cin/8 chunks, ntap taps); box = (8, npad, 2, box_taps):
-// box_taps consecutive taps' core-matrix planes (tap, half) of a 16-channel group in
-// one copy, laid out as [tap][half][npad][8] (mode 2 with split parities: the 8 taps
-// of one output row parity).
-bool encode_w4(CUtensorMap* m, const void* base, int cin, int npad, int ntap, int box_taps) {
-    const cuuint64_t dims[4] = {8u, (cuuint64_t)npad, (cuuint64_t)(cin / 8), (cuuint64_t)ntap};
-    const cuuint64_t strides[3] = {(cuuint64_t)ntap * cin * 2, 16u, (cuuint64_t)cin * 2};
-    const cuuint32_t box[4] = {8u, (cuuint32_t)npad, 2u, (cuuint32_t)box_taps};
-    const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-    const CUresult r = encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides,
-                                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
 // Mode 4: weights [npad][9][cin] viewed as a 5-D tensor (8 channels, npad rows,
 // 3 column taps, cin/8 chunks, 3 tap rows); box = (8, npad, 3, 2, 3) lands as
 // [dy][half][dx][npad][8], so that the B operand of tap row dy is 3 npad rows.
@@ -979,30 +960,6 @@ bool encode_w5(CUtensorMap* m, const void* base, int cin, int npad) {
     const cuuint32_t box[5] = {8u, (cuuint32_t)npad, 3u, 2u, 3u};
     const cuuint32_t estr[5] = {1u, 1u, 1u, 1u, 1u};
     return encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Mode 6: weights [npad][9][cin] viewed as a 5-D tensor (8 channels, npad rows, 3 tap
-// rows, cin/8 chunks, 3 column taps); box = (8, npad, 3, 2, 3) lands as [dx][half][dy][npad][8],
-// so that the B operand of column shift dx is 3 npad rows (dy, o).
-bool encode_w6(CUtensorMap* m, const void* base, int cin, int npad) {
-    const cuuint64_t dims[5] = {8u, (cuuint64_t)npad, 3u, (cuuint64_t)(cin / 8), 3u};
-    const cuuint64_t strides[4] = {(cuuint64_t)9 * cin * 2, (cuuint64_t)3 * cin * 2, 16u, (cuuint64_t)cin * 2};
-    const cuuint32_t box[5] = {8u, (cuuint32_t)npad, 3u, 2u, 3u};
-    const cuuint32_t estr[5] = {1u, 1u, 1u, 1u, 1u};
-    return encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// weights [npad][ntap * cin] viewed as 2-D; box = 8 input channels x npad rows.
-bool encode_w(CUtensorMap* m, const void* base, int cin, int npad, int ntap) {
-    const cuuint64_t dims[2] = {(cuuint64_t)ntap * cin, (cuuint64_t)npad};
-    const cuuint64_t strides[1] = {(cuuint64_t)ntap * cin * 2};
-    const cuuint32_t box[2] = {8u, (cuuint32_t)npad};
-    const cuuint32_t estr[2] = {1u, 1u};
-    return encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -1367,14 +1324,13 @@ int launch_cfg(const ConvArgs& a_in, cudaStream_t st, const TileCfg& t) {
     if ((reinterpret_cast<uintptr_t>(a.x0) & 15) || (a.c1 && (reinterpret_cast<uintptr_t>(a.x1) & 15)) ||
         (reinterpret_cast<uintptr_t>(a.w) & 15))
         return HELM_EINVAL;
-    // an up layer runs on its phase-merged weights
-    if (a.mode == 2 && (!a.wup || (reinterpret_cast<uintptr_t>(a.wup) & 15))) return HELM_EINVAL;
+    const void* wst = a.mode == 2 ? a.wup : a.wst;   // (an up layer runs on its phase-merged weights)
+    if (!wst || (reinterpret_cast<uintptr_t>(wst) & 15)) return HELM_EINVAL;
     Geometry g{};
     int mode = a.mode;
     if (plan_launch(a, t, false, &mode, &g) != HELM_OK) return HELM_EINVAL;
     alignas(64) CUtensorMap tmw;
-    if ((mode == 4 && !encode_w5(&tmw, a.w, a.c0 + a.c1, a.npad)) ||
-        ((mode == 5 || mode == 6) && !encode_w6(&tmw, a.w, a.c0 + a.c1, a.npad))) {
+    if (mode == 4 && !encode_w5(&tmw, a.w, a.c0 + a.c1, a.npad)) {
         // no weight map for the variant: the plain same-grid kernel
         if (plan_launch(a, t, true, &mode, &g) != HELM_OK) return HELM_EINVAL;
     }
@@ -1393,12 +1349,7 @@ int launch_cfg(const ConvArgs& a_in, cudaStream_t st, const TileCfg& t) {
     } else {
         tm1 = tm0;
     }
-    if (a.mode < 4) {
-        const void* wsrc = a.mode == 2 ? (const void*)a.wup : (const void*)a.w;
-        const int ntap = a.mode == 2 ? 16 : 9;
-        g.w4 = encode_w4(&tmw, wsrc, a.c0 + a.c1, a.npad, ntap, g.psplit ? 8 : ntap) ? 1 : 0;
-        if (!g.w4 && !encode_w(&tmw, wsrc, a.c0 + a.c1, a.npad, ntap)) return HELM_EINVAL;
-    }
+    if (a.mode != 4) tmw = tm0;   // (unused)
     switch (a.mode) {
         case 4: ++g_launch_narrow; return launch_mode<4>(tm0, tm1, tmw, a, g, st);
         case 5: return launch_mode<5>(tm0, tm1, tmw, a, g, st);
