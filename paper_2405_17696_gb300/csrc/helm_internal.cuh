@@ -401,4 +401,12 @@ bool stencil_tuning_on();
 int stencil_tuned_count();
 void stencil_tune_reset();
 
+// Whether a caller's array can be worked on as it is: memory of the current device, on 16 bytes.
+bool direct_array(const void* p);
+// Whether two arrays of `bytes` each have no byte in common.
+inline bool disjoint_arrays(const void* a, const void* b, size_t bytes) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x + bytes <= y || y + bytes <= x;
+}
+
 }  // namespace helm
