@@ -401,11 +401,23 @@ WgradGeom wgrad_plan(int mode, int c0, int c1, int npad, int hin, int win, int h
     }
     g.tw = tw;
     g.rows = rows;
+    // The taps in equal groups (the K tile stays that of the fullest group) when every CTA has an SM: those of
+    // the largest group bound the launch.  128 to 64 channels, 256 x 128, 16 images, one GB300, groups of 8 and
+    // 1 taps and of 5 and 4: 391 and 272 us.  With one CTA too many (three groups of 51 on 152 SMs) a light
+    // last group lets it start early: 128 to 128 channels, 128 x 64, 4, 4, 1 and 3, 3, 3: 74 and 104 us.
+    const int per_group = std::max(1, (sms + g.ngroups - 1) / g.ngroups);
+    if (per_group * g.ngroups <= sms) {
+        g.taps_per_group = (9 + g.ngroups - 1) / g.ngroups;
+        g.max_chunks = g.taps_per_group * g.cx;
+        g.stage = (g.max_chunks + g.gchunks) * g.plane;
+        cols = 32;
+        while (cols < (uint32_t)((g.max_chunks + 15) / 16 * npad)) cols <<= 1;
+        g.tmem_cols = cols;
+    }
     g.ns = (int)std::min<size_t>(WG_MAX_NS, (WG_SMEM_MAX - g.slack) / g.stage);
     g.tiles_x = (Wt + tw - 1) / tw;
     g.tiles_y = (Ht + rows - 1) / rows;
     g.ktiles = (long long)nb * g.tiles_x * g.tiles_y * g.phases;
-    const int per_group = std::max(1, (sms + g.ngroups - 1) / g.ngroups);
     g.splits = (int)std::max<long long>(1, std::min<long long>(g.ktiles, per_group));
     return g;
 }
