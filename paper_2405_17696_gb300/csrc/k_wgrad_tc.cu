@@ -107,38 +107,47 @@ __global__ void __launch_bounds__(WG_NT) wgrad_tc_kernel(const __grid_constant__
     const long long ntiles = g.ktiles > (long long)blockIdx.x ? (g.ktiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     const int gofs = g.max_chunks * g.plane;             // the g planes within a stage
 
-    // K tile k -> image b, tile origin on the tile grid, output parity
-    auto tile_of = [&](long long k, int& b, int& xs, int& ys, int& ph) {
-        long long t = (long long)blockIdx.x + k * gridDim.x;
-        ph = (int)(t % g.phases);
-        t /= g.phases;
-        const int tx = (int)(t % g.tiles_x);
-        t /= g.tiles_x;
-        const int ty = (int)(t % g.tiles_y);
-        b = (int)(t / g.tiles_y);
-        xs = tx * g.tw;
-        ys = ty * g.rows;
-    };
-
     if (warp == 4) {
         // ---------------- TMA producer ----------------
         if ((tid & 31) == 0) {
             const uint32_t tx = (uint32_t)((chunks + g.gchunks) * g.plane);
             bool ok = true;
+            // Stage, parity and tile (output parity, column, row, image) advance as counters: with 64-bit
+            // divisions this thread's own instructions bounded the kernel (16 to 16 channels, 1024 x 512, 16
+            // images, one GB300: 526 us, of which 330 stayed with nearly all copies and products left out; 403 now).
+            int s = 0;
+            uint32_t par = 1;   // of the stage's last release
+            int ph, tx0, ty0, b;
+            {
+                int t = (int)blockIdx.x;
+                ph = t % g.phases;
+                t /= g.phases;
+                tx0 = t % g.tiles_x;
+                t /= g.tiles_x;
+                ty0 = t % g.tiles_y;
+                b = t / g.tiles_y;
+            }
+            int dph, dtx, dty, db;   // gridDim.x tiles on
+            {
+                int t = (int)gridDim.x;
+                dph = t % g.phases;
+                t /= g.phases;
+                dtx = t % g.tiles_x;
+                t /= g.tiles_x;
+                dty = t % g.tiles_y;
+                db = t / g.tiles_y;
+            }
             long long k = 0;
             for (; k < ntiles && ok; ++k) {
-                const int s = (int)(k % g.ns);
-                const long long use = k / g.ns;
-                if (use > 0 && !wg_wait(&empty[s], (uint32_t)((use - 1) & 1), abort_v, 32)) { ok = false; break; }
-                int b, xs, ys, ph;
-                tile_of(k, b, xs, ys, ph);
+                if (k >= g.ns && !wg_wait(&empty[s], par, abort_v, 32)) { ok = false; break; }
+                const int xs = tx0 * g.tw, ys = ty0 * g.rows;
                 const int b1 = a.c1 ? (a.x1_map ? __ldg(a.x1_map + b) : (a.x1_bcast ? 0 : b)) : 0;
                 unsigned char* st = smem + (size_t)s * g.stage;
                 tc::mbar_arrive_expect_tx(&full[s], tx);
                 const int py = ph >> 1, px = ph & 1;
+                int dy = t0 / 3 - 1, dx = t0 % 3 - 1;
+                unsigned char* d0 = st;
                 for (int i = 0; i < ntap; ++i) {
-                    const int t = t0 + i, dy = t / 3 - 1, dx = t % 3 - 1;
-                    unsigned char* d0 = st + (size_t)(i * g.cx) * g.plane;
                     unsigned char* d1 = d0 + (size_t)g.cx0 * g.plane;
                     if (MODE == 0) {
                         tc::tma_load_4d(d0, &tm_x0, 2 * (xs + dx), ys + dy, 0, b, &full[s]);
@@ -151,11 +160,30 @@ __global__ void __launch_bounds__(WG_NT) wgrad_tc_kernel(const __grid_constant__
                         tc::tma_load_4d(d0, &tm_x0, 2 * (xs + fx), ys + fy, 0, b, &full[s]);
                         if (a.c1) tc::tma_load_4d(d1, &tm_x1, 2 * (xs + fx), ys + fy, 0, b1, &full[s]);
                     }
+                    d0 += (size_t)g.cx * g.plane;
+                    if (++dx == 2) {
+                        dx = -1;
+                        ++dy;
+                    }
                 }
                 if (MODE == 2)
                     tc::tma_load_5d(st + gofs, &tm_g, 0, 2 * xs + px, 2 * ys + py, 0, b, &full[s]);
                 else
                     tc::tma_load_4d(st + gofs, &tm_g, 2 * xs, ys, 0, b, &full[s]);
+                if (++s == g.ns) {
+                    s = 0;
+                    par ^= 1;
+                }
+                ph += dph;
+                int c = ph >= g.phases;
+                ph -= c ? g.phases : 0;
+                tx0 += dtx + c;
+                c = tx0 >= g.tiles_x;
+                tx0 -= c ? g.tiles_x : 0;
+                ty0 += dty + c;
+                c = ty0 >= g.tiles_y;
+                ty0 -= c ? g.tiles_y : 0;
+                b += db + c;
             }
             if (!ok) {
                 *abort_v = 1;
@@ -177,9 +205,10 @@ __global__ void __launch_bounds__(WG_NT) wgrad_tc_kernel(const __grid_constant__
         const uint32_t plane16 = (uint32_t)g.plane >> 4;
         const int ksteps = g.P / 16;
         bool ok = true;
+        int s = 0;
+        uint32_t par = 0;
         for (long long k = 0; k < ntiles && ok; ++k) {
-            const int s = (int)(k % g.ns);
-            const bool f_ok = wg_wait(&full[s], (uint32_t)((k / g.ns) & 1), abort_v, 32);
+            const bool f_ok = wg_wait(&full[s], par, abort_v, 32);
             if (!__all_sync(0xffffffffu, f_ok)) { ok = false; break; }
             tc::tc_fence_after_sync();
             const uint32_t s16 = (tc::smem_u32(smem + (size_t)s * g.stage) & 0x3FFFFu) >> 4;
@@ -197,6 +226,10 @@ __global__ void __launch_bounds__(WG_NT) wgrad_tc_kernel(const __grid_constant__
             }
             __syncwarp();
             if (leader) tc::mma_commit(&empty[s]);
+            if (++s == g.ns) {
+                s = 0;
+                par ^= 1;
+            }
         }
         if (!ok) *abort_v = 1;
         __syncwarp();
