@@ -42,6 +42,7 @@ struct WgradGeom {
     int stage, ns, slack;        // bytes per stage, stages, bytes after the ring
     uint32_t tmem_cols;
     int splits;                  // CTAs along K (gridDim.x)
+    int rows3;                   // same grid, one-row tiles, one group: planes [dx][chunk][dy], three rows a box
 };
 
 WgradGeom wgrad_plan(int mode, int c0, int c1, int npad, int hin, int win, int hout, int wout, int nb, int sms);
