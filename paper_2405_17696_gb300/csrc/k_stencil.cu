@@ -266,8 +266,11 @@ __global__ void zero_x_kernel(OuterState os, double2* x, size_t n) {
 
 int launch_apply_fine(const helm_ctx* c, const OpFine5& op, const float2* x, float2* y, int nb, const int* mask) {
     LaunchScope scope(c, K_APPLY);
-    // node pairs when the rows and the fields start on 16 bytes
-    if (op.nx % 2 == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0) {
+    // Node pairs when the rows and the fields start on 16 bytes, from 1.5 million nodes on: a pair's thread walks
+    // its rows one after another, which a launch that does not fill the SMs has to wait for.  A call on one
+    // GB300, a node and a pair per thread: 160 x 160 22.1 and 23.0 us, 512 x 256, 8 fields, 25.7 and 26.5,
+    // 16 fields 29.5 and 28.0, 32 fields 36.8 and 31.1.
+    if (op.nx % 2 == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 && (size_t)op.nx * op.nz * nb >= (3u << 19)) {
         const int xt = (op.nx / 2 + TILE_X - 1) / TILE_X, rows = arnoldi_rows(xt, op.nz, nb);
         { apply_fine2_kernel<<<dim3(xt, (op.nz + TILE_Y * rows - 1) / (TILE_Y * rows), nb), dim3(TILE_X, TILE_Y), 0, c->stream>>>(
             op, x, y, rows, mask, tally(c, K_APPLY, 16ull * op.nx * op.nz)); count_launch(); }
