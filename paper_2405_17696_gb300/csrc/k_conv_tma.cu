@@ -42,10 +42,8 @@
 //    serves all three (N = npad or 2 npad at the tile's ends).  A pixel is read by 3 MMAs instead
 //    of 9, and an output row still sums (group, dy, dx) in mode 0's order, bit for bit.  One MMA
 //    of zeros clears the tile's columns, since every other one adds to rows in progress.  Mode 0
-//    at 32 -> 16 channels spends 76 % of the cycles on operand reads; 1024 x 512, 32 images, one
-//    GB300, mode 0 and mode 5: 344 and 305 us for one layer of 16 channels;
-//    the 29 layers of a network pass took 7.41 ms and took 7.17 (5.04 with the epilogue below and
-//    the weights' contiguous copy).
+//    at 32 -> 16 channels spends 76 % of the cycles on operand reads.  1024 x 512, 32 images, one GB300:
+//    the 29 layers of a network pass 5.79 ms with mode 0 and 5.02 with mode 5 where rowsum_pays says so.
 //  6 (16 or 32 output channels, same grid as mode 0) the three tap rows in N: an M block is
 //    one staged row (pitch tw + 2 <= 128, lanes >= tw dropped) and per 16-channel group takes
 //    three MMAs, one per column shift dx, computing D[b][x][(dy, o)] for N = 3 npad.  Output
@@ -1166,8 +1164,11 @@ int mma_cycles(int n) { return std::max(n / 2, 32 + n / 4); }
 
 // Whether mode 5 (plan g5) takes fewer MMA cycles per output node and group than mode 0 (plan g0).  Mode
 // 5 reads A a third as often, but gives the lanes beyond a row's tile away (mode 0 packs rows), and its
-// tile ends carry fewer columns: 16 and 32 channels gain on every width that fills most of 128 lanes,
-// 64 channels have little to gain (their products already cost what A's reads do).
+// tile ends carry fewer columns.  The line lies a little below equal counts, where the two tie.  One GB300,
+// 32 images, mode 0 and mode 5 (modelled ratio): 16 channels, 1024 x 512, 220 and 163 us; 32 to 16 channels
+// there, 406 and 260; 32 channels, 512 x 256, 134 and 108; 64 channels, 512 x 64, 16 images, 59 and 50; 64
+// channels, 256 x 128, 199 and 198 (0.91); 32 channels, 128 x 64, 25 and 25 (1.00); 64 channels, 80 x 40, 28
+// and 33 (1.06); but 64 channels, 64 x 32, 28 and 24, which the count does not see.
 bool rowsum_pays(const ConvArgs& a, const Geometry& g0, const Geometry& g5) {
     if (g5.tiles <= 0 || 3 * a.npad > 256 || (size_t)g5.ns * g5.stage + ZERO_BYTES > 200 * 1024) return false;
     if (g0.tiles <= 0) return false;
