@@ -170,7 +170,9 @@ struct LegC9 {
 // Row rings in shared memory, filled by asynchronous copies AHEAD rows ahead.  A lane copies and reads
 // its own 16 bytes of a field's row; shared rows are copied by all warps and read after a barrier.
 // A copy into a slot is issued after row z's barrier (of the warp or the block), when every lane is
-// past row z - 1, so a ring holds rows z - 2 .. z + AHEAD.
+// past row z - 1, so a ring holds rows z - 2 .. z + AHEAD.  Rows after a march's last one are not copied, only
+// their empty groups are committed: the wait for the last row is then a wait for every copy of the march, and the
+// next frequency's march may fill the same slots (asynchronous copies to one address have no order).
 constexpr int AHEAD = 5, RING = 8;
 struct Ring {
     float4 row[RING][32];
@@ -250,10 +252,12 @@ __global__ void __launch_bounds__(32 * LEG_WARPS, LEG_CTAS) leg_down_kernel(L lo
         const bool mine = act && (!L::SHARED || freq == fq);
         lo.init(L::SHARED ? fq : freq);
         auto fetch = [&](int z) {
-            const bool in = col && z >= 0 && z < nz;
-            if (mine) copy16(&rf.row[z & (RING - 1)][lane], in ? fb + (size_t)z * nx : f, in);
-            for (int q = L::SHARED ? warp : 0; q < L::NCO; q += L::SHARED ? LEG_WARPS : 1)
-                copy16(&rm.row[z & (RING - 1)][q][lane], in ? lo.src(q, z * nx + 2 * k) : (const void*)f, in);
+            if (z <= z1 + 2) {
+                const bool in = col && z >= 0 && z < nz;
+                if (mine) copy16(&rf.row[z & (RING - 1)][lane], in ? fb + (size_t)z * nx : f, in);
+                for (int q = L::SHARED ? warp : 0; q < L::NCO; q += L::SHARED ? LEG_WARPS : 1)
+                    copy16(&rm.row[z & (RING - 1)][q][lane], in ? lo.src(q, z * nx + 2 * k) : (const void*)f, in);
+            }
             copy_commit();
         };
         for (int i = 0; i < AHEAD; ++i) fetch(z0 - 2 + i);
@@ -369,14 +373,16 @@ __global__ void __launch_bounds__(32 * LEG_WARPS, LEG_CTAS) leg_up_kernel(L lo, 
         };
         // row z with, for an even z, the coarse row z / 2 (which it and the odd row after it need)
         auto fetch = [&](int z) {
-            const bool in = col && z >= 0 && z < nz;
-            if (mine) {
-                copy16(&rf.row[z & (RING - 1)][lane], in ? fb + (size_t)z * nx : f, in);
-                copy16(&rv.row[z & (RING - 1)][lane], in ? vb + (size_t)z * nx : f, in);
-                if (!(z & 1)) fetch_e(z >> 1);
+            if (z <= z1 + 1) {
+                const bool in = col && z >= 0 && z < nz;
+                if (mine) {
+                    copy16(&rf.row[z & (RING - 1)][lane], in ? fb + (size_t)z * nx : f, in);
+                    copy16(&rv.row[z & (RING - 1)][lane], in ? vb + (size_t)z * nx : f, in);
+                    if (!(z & 1)) fetch_e(z >> 1);
+                }
+                for (int q = L::SHARED ? warp : 0; q < L::NCO; q += L::SHARED ? LEG_WARPS : 1)
+                    copy16(&rm.row[z & (RING - 1)][q][lane], in ? lo.src(q, z * nx + 2 * k) : (const void*)f, in);
             }
-            for (int q = L::SHARED ? warp : 0; q < L::NCO; q += L::SHARED ? LEG_WARPS : 1)
-                copy16(&rm.row[z & (RING - 1)][q][lane], in ? lo.src(q, z * nx + 2 * k) : (const void*)f, in);
             copy_commit();
         };
         // coarse row J at columns k - 1 and k
