@@ -8,19 +8,22 @@
 // neighbour CTA's halo (distributed shared memory), the inner products into every CTA.
 //
 // The basis is kept unnormalised: A v_j = sum_i (d_ij / n_i^2) v_i + v_{j+1} / ie_j with
-// d_ij = <v_i, A v_j> and n_i = ||v_i||, where ie_j = 1 / ||A v_j|| only sets the scale
-// v_{j+1} is stored at (no drift from step to step).  n_j^2 is reduced together
-// with the inner products of step j, so a step takes one reduction: FP32 within a
-// thread's strip and its warp, then two-term (hi + lo) sums over warps and CTAs.  The
-// (k+1) x k least-squares problem with columns d_ij / n_i, n_{j+1} / ie_j is solved in
-// two-term arithmetic at the end, each rotation applied to all later columns at once.
+// d_ij = <v_i, A v_j> and n_i = ||v_i||, where the power of two ie_j near 1 / ||A v_j|| only sets
+// the scale v_{j+1} is stored at (no drift from step to step, no rounding).  n_j^2 is reduced
+// together with the inner products of step j, so a step takes one reduction: FP32 within a
+// thread's strip, three-term sums, as good as FP64 ones (reduce.cuh), over lanes, warps and CTAs.
+// The (k+1) x k least-squares problem is solved in FP64 at the end, by rotations without square
+// roots (see there).
 //
 // Bound by latency: a step is two barriers, two sums and some 25 instructions per node and
 // basis vector.  Ten steps on one GB300, against one 512-thread block per right-hand side
 // with its vectors in L2 (k_coarse.cu, whose FP64 shuffle sums alone took about half):
-// 40 x 40, 1 RHS 269 -> 41 us; 128 x 64, 192 RHS 734 -> 334 us (32 clusters of four CTAs at a
-// time); 256 x 128, 16 RHS 1152 -> 184 us (sixteen CTAs); 340 x 172, 40 RHS 2636 -> 1470 us
-// (spilled vectors, coefficients from L2).
+// 40 x 40, 1 RHS 269 -> 45 us; 128 x 64, 192 RHS 734 -> 384 us (32 clusters of four CTAs at a
+// time); 256 x 128, 16 RHS 1152 -> 213 us (sixteen CTAs); 340 x 172, 40 RHS 2636 -> 1408 us
+// (spilled vectors, coefficients from L2).  With FP32 sums in a warp, two-term ones beyond and a two-term
+// least-squares solve it was 41, 336, 187 and 1368 us.  Error of V-cycles against 64 bits, the
+// mean over 24 grids for 4, 10 and 16 steps, as a multiple of that block's: 0.96, 0.96, 0.95 (0.99,
+// 0.99, 1.00 with those sums).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -50,19 +53,33 @@ struct CoarsePlan {
     size_t smem = 0;
 };
 
+// The power of two that takes a vector of squared norm x > 0 to a norm in [1, 2).
+__device__ __forceinline__ float pow2_rsqrt(float x) {
+    const int e = (int)(__float_as_uint(x) >> 23) - 127;
+    return __uint_as_float((unsigned)(127 - (e >> 1)) << 23);
+}
+
 template <int NPT, bool SPILL>
 __global__ void __launch_bounds__(SPILL ? 32 * CC_WARPS : 512)
 coarse_cluster_kernel(OpC9 op, const float2* __restrict__ f, float2* __restrict__ u, float2* __restrict__ V,
                       size_t vstride, int kmax, int S, int C, int nsm, const int* mask, Tally tl) {
     extern __shared__ __align__(16) unsigned char dynsm[];
-    __shared__ float2 redw[CC_WARPS][20];
-    __shared__ float4 part[CC_MAX][KMAX + 2];
-    __shared__ float4 hist[KMAX][KMAX + 1];         // d_ij as (re hi, re lo, im hi, im lo)
-    __shared__ float2 n2h[KMAX + 1], qs[KMAX + 1];  // n_j^2 and 1 / n_j^2 (hi, lo)
+    // the warps' sums of a step and, once the steps are done, the least-squares columns
+    __shared__ union Work {
+        float2 redw[3][CC_WARPS][20];               // terms (re, im) of a value per warp
+        struct {
+            double2 D[KMAX + 1][KMAX + 1], T[KMAX + 1][KMAX];   // columns, the right-hand side last
+            double2 a[KMAX];
+            double n2[KMAX + 1], u[KMAX];
+        } ls;
+    } wk;
+    __shared__ tf2 part[CC_MAX][KMAX + 2];
+    __shared__ tf2 hist[KMAX][KMAX + 1];            // d_ij
+    __shared__ tf n2h[KMAX + 1];                    // n_j^2
+    __shared__ float2 qs[KMAX + 1];                 // 1 / n_j^2 (hi, lo)
     __shared__ float ieh[KMAX];
-    __shared__ float4 Hs[KMAX + 1][KMAX + 3];       // least-squares columns, the right-hand side last
-    __shared__ float2 nsh[KMAX + 1], rns[KMAX + 1]; // n_j and 1 / n_j
     __shared__ float2 cfs[KMAX + 1];
+    __shared__ unsigned wmax[CC_WARPS], cmax[CC_MAX];
     __shared__ float ie_s;
     __shared__ int stop_s;
 
@@ -107,59 +124,64 @@ coarse_cluster_kernel(OpC9 op, const float2* __restrict__ f, float2* __restrict_
         v[m] = own && z0 + m < nz ? f[(size_t)b * n + (size_t)(z0 + m) * nx + ix] : make_float2(0.f, 0.f);
     for (int i = t; i < 2 * nx; i += blockDim.x) htop[i] = make_float2(0.f, 0.f);
 
-    // Sum nv complex values over the cluster, the caller having each warp's sums in redw: warp k sums
-    // value k (k + nwarp, ...) over the CTA's warps with a shuffle tree of two-term adds, sends it to
-    // every CTA, and after the cluster barrier sums the CTAs' values the same way.  use(k, value) runs
-    // in every lane of that warp.  The values pass through entries at .. at + nv - 1 of `part`; a sum
+    // Sum nv complex values over the cluster, the caller having each warp's sums in redw: groups of `wide`
+    // lanes (which cover the warps and, since lane c sends the sum to CTA c, the CTAs) take a value
+    // each, sum it over the CTA's warps with a shuffle tree of three-term adds, send it to every CTA,
+    // and after the cluster barrier sum the CTAs' values the same way.  use(k, value) runs in the first
+    // lane of a value's group.  The values pass through entries at .. at + nv - 1 of `part`; a sum
     // whose entries may still be read takes others (the last one, which no halo barrier separates
     // from the one before).
-    auto tree = [&](float4 r, int width) -> float4 {
-        for (int o = width >> 1; o > 0; o >>= 1) {
-            const ff x = ff_add({r.x, r.y}, {__shfl_xor_sync(0xffffffffu, r.x, o), __shfl_xor_sync(0xffffffffu, r.y, o)});
-            const ff y = ff_add({r.z, r.w}, {__shfl_xor_sync(0xffffffffu, r.z, o), __shfl_xor_sync(0xffffffffu, r.w, o)});
-            r = make_float4(x.h, x.l, y.h, y.l);
-        }
-        return r;
-    };
-    // tree widths: cwide covers the CTAs; wwide the warps and, since lane c sends the sum to CTA c, the CTAs
-    int cwide = 1;
-    while (cwide < C) cwide <<= 1;
-    int wwide = cwide;
-    while (wwide < nwarp) wwide <<= 1;
+    // (a spilling CTA has more than eight warps: fixed there, which keeps registers.)
+    int wide = SPILL ? 32 : 1;
+    while (!SPILL && (wide < C || wide < nwarp)) wide <<= 1;
+    const int sub = lane & (wide - 1), k0 = (warp * 32 + lane) / wide, kstep = nwarp * 32 / wide;
+    const tf2 none = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     auto cluster_sum = [&](int nv, int at, auto use) {
         __syncthreads();
-        for (int k = warp; k < nv; k += nwarp) {
-            const float2 x = lane < nwarp ? redw[lane][k] : make_float2(0.f, 0.f);
-            const float4 r = tree(make_float4(x.x, 0.f, x.y, 0.f), wwide);
-            if (C == 1) use(k, r);
-            else if (lane < C) *cl.map_shared_rank(&part[rank][at + k], lane) = r;
+        for (int kb = warp * 32 / wide, k = k0; kb < nv; kb += kstep, k += kstep) {
+            tf2 x = none;
+            if (sub < nwarp && k < nv) x = {wk.redw[0][sub][k], wk.redw[1][sub][k], wk.redw[2][sub][k]};
+            x = tf2_group_sum(x, wide);
+            if (k >= nv) continue;
+            if (C == 1) {
+                if (sub == 0) use(k, x);
+            } else if (sub < C) {
+                *cl.map_shared_rank(&part[rank][at + k], sub) = x;
+            }
         }
         if (C == 1) return;
         sync_all();
-        for (int k = warp; k < nv; k += nwarp)
-            use(k, tree(lane < C ? part[lane][at + k] : make_float4(0.f, 0.f, 0.f, 0.f), cwide));
+        for (int kb = warp * 32 / wide, k = k0; kb < nv; kb += kstep, k += kstep) {
+            const tf2 x = tf2_group_sum(sub < C && k < nv ? part[sub][at + k] : none, wide);
+            if (sub == 0 && k < nv) use(k, x);
+        }
     };
 
-    // beta = ||f||: v_0 = f / beta (in FP32; n_0 below is the exact norm of what is stored)
+    // v_0 = f inv0 with a power of two that takes the largest component to about 1 / sqrt(n), so that ||v_0|| is at
+    // most about 2 (n_0 below is the norm of what is stored).  Zero, infinite or NaN f: u = 0.
+    float inv0;
     {
-        float a = 0.f;
-#pragma unroll
-        for (int m = 0; m < NPT; ++m) a += v[m].x * v[m].x + v[m].y * v[m].y;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) redw[warp][0] = make_float2(a, 0.f);
-        if (C > 1) sync_all();                       // every CTA of the cluster runs: remote stores may start
-        cluster_sum(1, 0, [&](int, const float4& r) {
-            if (lane == 0) ie_s = r.x > 0.f && isfinite(r.x) ? rsqrtf(r.x) : 0.f;
-        });
-        __syncthreads();
-    }
-    const float inv0 = ie_s;
-    if (!(inv0 > 0.f)) {
+        unsigned a = 0u;
 #pragma unroll
         for (int m = 0; m < NPT; ++m)
-            if (own && z0 + m < nz) u[(size_t)b * n + (size_t)(z0 + m) * nx + ix] = make_float2(0.f, 0.f);
-        return;
+            a = max(a, max(__float_as_uint(v[m].x) & 0x7fffffffu, __float_as_uint(v[m].y) & 0x7fffffffu));
+        a = __reduce_max_sync(0xffffffffu, a);
+        if (lane == 0) wmax[warp] = a;
+        sync_all();                                  // (every CTA of the cluster runs: remote stores may start)
+        a = __reduce_max_sync(0xffffffffu, lane < nwarp ? wmax[lane] : 0u);
+        if (C > 1) {
+            if (warp == 0 && lane < C) *cl.map_shared_rank(&cmax[rank], lane) = a;
+            sync_all();
+            a = __reduce_max_sync(0xffffffffu, lane < C ? cmax[lane] : 0u);
+        }
+        if (a == 0u || a >= 0x7f800000u) {
+#pragma unroll
+            for (int m = 0; m < NPT; ++m)
+                if (own && z0 + m < nz) u[(size_t)b * n + (size_t)(z0 + m) * nx + ix] = make_float2(0.f, 0.f);
+            return;
+        }
+        const int e = 254 - (int)(a >> 23) - (31 - __clz(n)) / 2;
+        inv0 = __uint_as_float((unsigned)min(max(e, 1), 253) << 23);
     }
 #pragma unroll
     for (int m = 0; m < NPT; ++m) v[m] = cscale(inv0, v[m]);
@@ -259,45 +281,31 @@ coarse_cluster_kernel(OpC9 op, const float2* __restrict__ f, float2* __restrict_
                         a[2 * q + 1] = ay;
                     }
             }
-            // eight warp sums in nine shuffles: each halving step leaves a lane with half the values
-            float h4[4], h2[2], h1;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float keep = lane & 16 ? a[k + 4] : a[k], give = lane & 16 ? a[k] : a[k + 4];
-                h4[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+            const tf h = tf_warp_sum8(a, lane);
+            if ((lane & 3) == 0) {                    // value lane >> 2 of the eight
+                reinterpret_cast<float*>(&wk.redw[0][warp][i0])[lane >> 2] = h.h;
+                reinterpret_cast<float*>(&wk.redw[1][warp][i0])[lane >> 2] = h.m;
+                reinterpret_cast<float*>(&wk.redw[2][warp][i0])[lane >> 2] = h.l;
             }
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const float keep = lane & 8 ? h4[k + 2] : h4[k], give = lane & 8 ? h4[k] : h4[k + 2];
-                h2[k] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
-            }
-            {
-                const float keep = lane & 4 ? h2[1] : h2[0], give = lane & 4 ? h2[0] : h2[1];
-                h1 = keep + __shfl_xor_sync(0xffffffffu, give, 4);
-            }
-            h1 += __shfl_xor_sync(0xffffffffu, h1, 2);
-            h1 += __shfl_xor_sync(0xffffffffu, h1, 1);
-            if ((lane & 3) == 0)                      // value 4 bit4 + 2 bit3 + bit2 of the eight
-                reinterpret_cast<float*>(&redw[warp][i0])[lane >> 2] = h1;
         }
         // the last value carries n_j^2 and ||w||^2; c_i = d_ij / n_i^2 waits for 1 / n_j^2 only at i = j
-        cluster_sum(nv, j < kmax ? 0 : KMAX + 1, [&](int k, const float4& d) {
-            if (lane != 0) return;
+        // (c_i is an FP32 factor: two-term numbers on the way to it)
+        cluster_sum(nv, j < kmax ? 0 : KMAX + 1, [&](int k, const tf2& d) {
             if (k == nv - 1) {
-                n2h[j] = make_float2(d.z, d.w);
-                stop_s = j == kmax || !(d.z > 0.f) || !isfinite(d.z) ? 1 : 0;
+                n2h[j] = second_of(d);
+                stop_s = j == kmax || !(d.h.y > 0.f) || !isfinite(d.h.y) ? 1 : 0;
                 if (j < kmax) {
-                    const float ie = d.x > 0.f ? rsqrtf(d.x) : 1.f;
+                    const float ie = d.h.x > 0.f ? pow2_rsqrt(d.h.x) : 1.f;
                     ie_s = ie;
                     ieh[j] = ie;
                 }
-                const ff q = ff_rcp({d.z, d.w});
+                const ff q = ff_rcp({d.h.y, d.m.y});
                 qs[j] = make_float2(q.h, q.l);
             } else {
                 hist[j][k] = d;
                 if (k < j) {
                     const ff q = {qs[k].x, qs[k].y};
-                    cfs[k] = make_float2(ff_mul({d.x, d.y}, q).h, ff_mul({d.z, d.w}, q).h);
+                    cfs[k] = make_float2(ff_mul({d.h.x, d.m.x}, q).h, ff_mul({d.h.y, d.m.y}, q).h);
                 }
             }
         });
@@ -313,9 +321,9 @@ coarse_cluster_kernel(OpC9 op, const float2* __restrict__ f, float2* __restrict_
                 if (i < j) {
                     c = cfs[i];
                 } else {
-                    const float4 d = hist[j][j];
+                    const tf2 d = hist[j][j];
                     const ff q = {qs[j].x, qs[j].y};
-                    c = make_float2(ff_mul({d.x, d.y}, q).h, ff_mul({d.z, d.w}, q).h);
+                    c = make_float2(ff_mul({d.h.x, d.m.x}, q).h, ff_mul({d.h.y, d.m.y}, q).h);
                 }
                 if (!SPILL || i < nsm) {
                     const float2* vp = slots + (size_t)i * slab + loc;
@@ -342,73 +350,94 @@ coarse_cluster_kernel(OpC9 op, const float2* __restrict__ f, float2* __restrict_
         for (int m = 0; m < NPT; ++m) v[m] = cscale(ie, w[m]);
     }
 
-    // least squares min || beta e_1 - H y ||: lane c < steps has column c, lane `steps` the right-hand side
-    if (warp == 0) {
+    // Least squares in FP64: min || f inv0 - sum_c y_c ie_c A v_c ||, of which row i of column c is D[c][i] =
+    // <v_i, ie_c A v_c> with weight 1 / n_i^2; its subdiagonal entry is n_{c+1}^2, the right-hand side (n_0^2, 0, ..).
+    // Rotation i takes the running row t (entries T[c][i], a = T[i][i], weight 1 / u_i) and row i + 1, q, with h =
+    // n_{i+1}^2, to the pivot row b = h conj(a) t + u_i h q, whose own entry is u_{i+1} = h |a|^2 + h^2 u_i, and the next
+    // running row a q - h t of weight 1 / u_{i+1}: Givens rotations without their roots and quotients (Gentleman 1973).
+    // An FP64 instruction takes a warp 64 cycles, so those off the chain run on other warps or once for all rows
+    // (by Givens rotations in one warp this took 18 us for ten steps).
+    {
         const int m = steps;
-        if (lane <= m) {
-            const ff n2 = {n2h[lane].x, n2h[lane].y};
-            const ff r = n2.h > 0.f ? ff_rsqrt(n2) : ff{0.f, 0.f}, nn = ff_mul(n2, r);
-            rns[lane] = make_float2(r.h, r.l);
-            nsh[lane] = make_float2(nn.h, nn.l);
+        auto& ls = wk.ls;
+        auto wide2 = [](const tf& s) { return (widen(s.l) + widen(s.m)) + widen(s.h); };
+        for (int e = t, c = 0, c0 = 0; e < m * (m + 1) / 2; e += blockDim.x) {   // entries i <= c
+            while (e > c0 + c) c0 += ++c;
+            const tf2 d = hist[c][e - c0];
+            const double s = ieh[c];
+            ls.D[c][e - c0] = make_double2(wide2(first_of(d)) * s, wide2(second_of(d)) * s);
         }
-        __syncwarp();
-        if (lane < m) {
-            for (int i = 0; i <= lane; ++i) {
-                const float4 d = hist[lane][i];
-                const ff rn = {rns[i].x, rns[i].y}, x = ff_mul(ff{d.x, d.y}, rn), y = ff_mul(ff{d.z, d.w}, rn);
-                Hs[lane][i] = make_float4(x.h, x.l, y.h, y.l);
-            }
-            const ff x = ff_mul(ff{nsh[lane + 1].x, nsh[lane + 1].y}, ff_rcp(ff{ieh[lane], 0.f}));
-            Hs[lane][lane + 1] = make_float4(x.h, x.l, 0.f, 0.f);
-        } else if (lane == m) {
-            const ff x = ff_mul(ff{nsh[0].x, nsh[0].y}, ff_rcp(ff{inv0, 0.f}));
-            Hs[m][0] = make_float4(x.h, x.l, 0.f, 0.f);
-            for (int i = 1; i <= m; ++i) Hs[m][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t <= m) {
+            const double h = wide2(n2h[t]);
+            ls.n2[t] = h;
+            ls.D[m][t] = make_double2(t == 0 ? h : 0.0, 0.0);
         }
-        __syncwarp();
-        ff rinv = {0.f, 0.f};                         // lane i: 1 / R_ii
-        float4 p = lane <= m ? Hs[lane][0] : make_float4(0.f, 0.f, 0.f, 0.f);   // row i of this lane's column
-        for (int i = 0; i < m; ++i) {
-            ff cx = {0.f, 0.f}, cy = {0.f, 0.f}, sn = {0.f, 0.f};
-            if (lane == i) {
-                const ff ax = {p.x, p.y}, ay = {p.z, p.w}, hb = {Hs[i][i + 1].x, Hs[i][i + 1].y};
-                const ff x = ff_add(ff_add(ff_mul(ax, ax), ff_mul(ay, ay)), ff_mul(hb, hb));
-                // (x = 0: no component; x not finite: it stays so)
-                rinv = x.h > 0.f ? ff_rsqrt(x) : x;
-                cx = ff_mul(ax, rinv);
-                cy = ff_mul(ay, rinv);
-                sn = ff_mul(hb, rinv);
+        __syncthreads();
+        double piv = 0.0;                             // lane i of warp 0: u_{i+1}
+        const int col = lane / 2 + 1;                 // lanes 2 c - 2 and 2 c - 1: the parts of column c
+        const bool im = lane & 1;
+        if (warp == 0) {
+            double tc = 0.0, ax = 0.0, ay = 0.0;
+            if (col <= m) tc = im ? ls.D[col][0].y : ls.D[col][0].x;
+            for (int i = 0; i < m; ++i) {
+                double px = __shfl_sync(0xffffffffu, tc, 2 * i - 2 & 31), py = __shfl_sync(0xffffffffu, tc, 2 * i - 1 & 31);
+                if (i == 0) {
+                    px = ls.D[0][0].x;
+                    py = ls.D[0][0].y;
+                }
+                if (lane == i) {
+                    ax = px;
+                    ay = py;
+                }
+                if (col > i && col <= m) {
+                    const double2 q = ls.D[col][i + 1];
+                    reinterpret_cast<double*>(&ls.T[col][i])[im] = tc;
+                    tc = fma(px, im ? q.y : q.x, fma(im ? py : -py, im ? q.x : q.y, -ls.n2[i + 1] * tc));
+                }
             }
-            cx = ff_shfl(cx, i);
-            cy = ff_shfl(cy, i);
-            sn = ff_shfl(sn, i);
-            if (lane > i && lane <= m) {              // [conj(c) s; -s c] on rows i, i + 1
-                const float4 q = Hs[lane][i + 1];
-                const ff px = {p.x, p.y}, py = {p.z, p.w}, qx = {q.x, q.y}, qy = {q.z, q.w};
-                const ff tx = ff_add(ff_add(ff_mul(cx, px), ff_mul(cy, py)), ff_mul(sn, qx));
-                const ff ty = ff_add(ff_add(ff_mul(cx, py), ff_neg(ff_mul(cy, px))), ff_mul(sn, qy));
-                const ff vx = ff_add(ff_add(ff_mul(cx, qx), ff_neg(ff_mul(cy, qy))), ff_neg(ff_mul(sn, px)));
-                const ff vy = ff_add(ff_add(ff_mul(cx, qy), ff_mul(cy, qx)), ff_neg(ff_mul(sn, py)));
-                Hs[lane][i] = make_float4(tx.h, tx.l, ty.h, ty.l);
-                p = make_float4(vx.h, vx.l, vy.h, vy.l);
+            const double h = lane < m ? ls.n2[lane + 1] : 0.0, hx = h * ax, hy = h * ay, w = fma(hx, ax, hy * ay), hh = h * h;
+            double u = ls.n2[0], uo = 0.0;
+            for (int i = 0; i < m; ++i) {
+                if (lane == i) uo = u;
+                u = fma(__shfl_sync(0xffffffffu, hh, i), u, __shfl_sync(0xffffffffu, w, i));
+                if (lane == i) piv = u;
+            }
+            if (lane < m) {
+                ls.a[lane] = make_double2(hx, hy);
+                ls.u[lane] = uo * h;
             }
         }
-        __syncwarp();
-        ff gx = {0.f, 0.f}, gy = {0.f, 0.f};
-        if (lane < m) {
-            const float4 g = Hs[m][lane];
-            gx = {g.x, g.y};
-            gy = {g.z, g.w};
-        }
-        for (int c = m - 1; c >= 0; --c) {
-            const ff yx = ff_shfl(ff_mul(gx, rinv), c), yy = ff_shfl(ff_mul(gy, rinv), c);
-            if (lane < c) {
-                const float4 r = Hs[c][lane];
-                const ff rx = ff_neg(ff{r.x, r.y}), ry = ff_neg(ff{r.z, r.w});
-                gx = ff_add(ff_add(gx, ff_mul(rx, yx)), ff_neg(ff_mul(ry, yy)));
-                gy = ff_add(ff_add(gy, ff_mul(rx, yy)), ff_mul(ry, yx));
+        __syncthreads();
+        // the pivot rows over T while warp 0 takes the reciprocals of their own entries
+        if (warp == 0) {
+            // (0: no component; not finite: it stays so)
+            piv = piv > 0.0 ? 1.0 / piv : piv;
+        } else {
+            for (int e = t - 32, c = 1, c0 = 0; e < m * (m + 1) / 2; e += blockDim.x - 32) {   // entries i < c <= m
+                while (e >= c0 + c) c0 += c++;
+                const int i = e - c0;
+                const double2 a = ls.a[i], b = ls.T[c][i], q = ls.D[c][i + 1];
+                const double w = ls.u[i];
+                ls.T[c][i] = make_double2(fma(a.x, b.x, fma(a.y, b.y, w * q.x)), fma(a.x, b.y, fma(-a.y, b.x, w * q.y)));
             }
-            if (lane == c) cfs[c] = make_float2(yx.h, yy.h);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // back substitution: lanes 2 i and 2 i + 1 have the parts of row i
+            const int row = lane / 2;
+            const double r = __shfl_sync(0xffffffffu, piv, row);
+            double g = 0.0;
+            if (row < m) g = im ? ls.T[m][row].y : ls.T[m][row].x;
+            for (int c = m - 1; c >= 0; --c) {
+                const double y = g * r, yx = __shfl_sync(0xffffffffu, y, 2 * c), yy = __shfl_sync(0xffffffffu, y, 2 * c + 1);
+                if (row < c) {
+                    const double2 b = ls.T[c][row];
+                    g = fma(-b.x, im ? yy : yx, fma(im ? -b.y : b.y, im ? yx : yy, g));
+                } else if (lane == 2 * c) {
+                    const double s = (double)ieh[c] * (double)(1.0f / inv0);   // powers of two
+                    cfs[c] = make_float2((float)(yx * s), (float)(yy * s));
+                }
+            }
         }
     }
     __syncthreads();

@@ -75,22 +75,6 @@ __global__ void __launch_bounds__(NTHREADS) apply_fine2_kernel(OpFine5 op, const
     }
 }
 
-// float <-> double by integer operations: conversions run at the FP64 pipe's two per SM and cycle, which
-// bounds the residual below.  Zeros, denormals, infinities and NaN take the instruction.
-__device__ __forceinline__ double widen(float f) {
-    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
-    if (e - 1u >= 254u) return (double)f;
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
-}
-// round to nearest even
-__device__ __forceinline__ float narrow(double d) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
-    const unsigned e = (unsigned)(u >> 52) & 0x7ffu;
-    if (e - 897u >= 253u) return (float)d;            // (the largest finite exponent too: it may round up to infinity)
-    const unsigned long long v = u + 0x0fffffffull + ((u >> 29) & 1ull);
-    return __uint_as_float(((unsigned)(u >> 32) & 0x80000000u) | ((unsigned)((v >> 29) & 0xffffffffull) - (896u << 23) & 0x7fffffffu));
-}
-
 // r = b - H x evaluated in FP64 from the complex128 iterate x (b conjugated
 // when solving the adjoint system); r is stored in complex64 as the first
 // (unscaled) Krylov vector.  ||r||^2 and, on the first call, ||b||^2 are
