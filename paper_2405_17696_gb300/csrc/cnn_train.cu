@@ -447,12 +447,11 @@ int layer_wgrad(const __nv_bfloat16* x0, int c0, const __nv_bfloat16* x1, int c1
     const unsigned gy = (unsigned)((c0 + c1 + 15) / 16), gz = (unsigned)(npad / 16);
     const long long tiles = (long long)nb * w.tiles_x * w.tiles_y;
     const long long gx = std::max<long long>(1, std::min<long long>(tiles, 1216 / (gy * gz)));
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        attr = true;
-    }
+    static DeviceOnce once;
+    HELM_CK(once_per_device(once, [] {
+        const cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    }));
     LaunchScope scope(prof_ctx, K_WGRAD);
     { wgrad_kernel<<<dim3((unsigned)gx, gy, gz), 256, smem, st>>>(a, w); count_launch(); }
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_ECUDA;

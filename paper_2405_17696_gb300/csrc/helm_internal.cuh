@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "device_once.h"
 #include "helm.h"
 
 namespace helm {
@@ -400,6 +401,14 @@ void stencil_tuning(bool on);
 bool stencil_tuning_on();
 int stencil_tuned_count();
 void stencil_tune_reset();
+
+// set() (a cudaError_t) once on every device that gets here, see DeviceOnce.
+template <class F>
+cudaError_t once_per_device(DeviceOnce& once, F set) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : (cudaError_t)once.run(dev, [&] { return (int)set(); });
+}
 
 // Whether a caller's array can be worked on as it is: memory of the current device, on 16 bytes.
 bool direct_array(const void* p);

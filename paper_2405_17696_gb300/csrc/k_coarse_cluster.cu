@@ -466,16 +466,14 @@ coarse_cluster_kernel(OpC9 op, const float2* __restrict__ f, float2* __restrict_
 
 template <int NPT, bool SPILL>
 bool cc_attributes() {
-    static std::once_flag once;
-    static bool ok = false;
-    std::call_once(once, [] {
-        ok = cudaFuncSetAttribute(coarse_cluster_kernel<NPT, SPILL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)CC_SMEM) == cudaSuccess &&
-             cudaFuncSetAttribute(coarse_cluster_kernel<NPT, SPILL>, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                                  1) == cudaSuccess;
-        (void)cudaGetLastError();
+    static DeviceOnce once;
+    const cudaError_t e = once_per_device(once, [] {
+        const cudaError_t s = cudaFuncSetAttribute(coarse_cluster_kernel<NPT, SPILL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC_SMEM);
+        return s != cudaSuccess ? s : cudaFuncSetAttribute(coarse_cluster_kernel<NPT, SPILL>,
+                                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     });
-    return ok;
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e == cudaSuccess;
 }
 
 void cc_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, const CoarsePlan& p, int nb, cudaStream_t st) {

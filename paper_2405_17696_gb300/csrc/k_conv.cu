@@ -257,11 +257,10 @@ __global__ void __launch_bounds__(NT) conv3x3_tc_kernel(ConvArgs a) {
 template <int CK>
 int launch_ck(const ConvArgs& a, cudaStream_t st) {
     const size_t smem = (size_t)ns_of(CK) * 2 * CT * CK * 2;
-    static bool configured = false;   // attribute is per function; setting it twice is harmless
-    if (!configured) {
-        cudaFuncSetAttribute(conv3x3_tc_kernel<CK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        configured = true;
-    }
+    static DeviceOnce once;
+    HELM_CK(once_per_device(once, [&] {
+        return cudaFuncSetAttribute(conv3x3_tc_kernel<CK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }));
     const long long mtot = (long long)a.nb * a.hout * a.wout;
     const unsigned grid = (unsigned)((mtot + CT - 1) / CT);
     { conv3x3_tc_kernel<CK><<<grid, NT, smem, st>>>(a); count_launch(); }

@@ -1211,12 +1211,12 @@ int sm_count() {
 template <int MODE, bool ACT>
 int launch_kernel(const CUtensorMap& tm0, const CUtensorMap& tm1, const CUtensorMap& tmw, const ConvArgs& a,
                 const Geometry& g, cudaStream_t st) {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(conv3x3_tma_kernel<MODE, ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    static DeviceOnce once;
+    HELM_CK(once_per_device(once, [] {
+        const cudaError_t e = cudaFuncSetAttribute(conv3x3_tma_kernel<MODE, ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         // all of the unified L1/shared storage as shared memory: two CTAs of ~100 KB per SM
-        cudaFuncSetAttribute(conv3x3_tma_kernel<MODE, ACT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    });
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(conv3x3_tma_kernel<MODE, ACT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    }));
     const size_t smem = (size_t)g.ns * g.stage;
     // two CTAs per SM when two fit the 512 TMEM columns, else one; a shared-memory
     // request above a third (half) of the SM keeps further CTAs off

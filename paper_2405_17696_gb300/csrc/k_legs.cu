@@ -23,7 +23,6 @@
 // right-hand sides), so every warp reads its own.
 #include <algorithm>
 #include <cstdint>
-#include <mutex>
 #include <type_traits>
 
 #include "helm_internal.cuh"
@@ -470,14 +469,12 @@ constexpr size_t LEG_UP_SMEM = COEF_RINGS<L> * sizeof(Coefs<L>) + LEG_WARPS * (2
 
 template <class L>
 int leg_attributes() {
-    static std::once_flag once;
-    static cudaError_t e = cudaSuccess;
-    std::call_once(once, [] {
-        e = cudaFuncSetAttribute(leg_down_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LEG_DOWN_SMEM<L>);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(leg_up_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LEG_UP_SMEM<L>);
-    });
-    HELM_CK(e);
+    static DeviceOnce once;
+    HELM_CK(once_per_device(once, [] {
+        const cudaError_t e = cudaFuncSetAttribute(leg_down_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LEG_DOWN_SMEM<L>);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(leg_up_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)LEG_UP_SMEM<L>);
+    }));
     return HELM_OK;
 }
 

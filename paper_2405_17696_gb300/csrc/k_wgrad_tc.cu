@@ -390,11 +390,11 @@ int sm_count_wg() {
 template <int MODE>
 int launch_wg_mode(const CUtensorMap& tx0, const CUtensorMap& tx1, const CUtensorMap& tg, const WgradArgs& a,
                    const WgradGeom& g, cudaStream_t st) {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(wgrad_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM_MAX);
-        cudaFuncSetAttribute(wgrad_tc_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    });
+    static DeviceOnce once;
+    HELM_CK(once_per_device(once, [] {
+        const cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM_MAX);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(wgrad_tc_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    }));
     // at least 116 KB, so that one CTA per SM holds the TMEM (up to all 512 columns)
     const size_t smem = std::max<size_t>((size_t)g.ns * g.stage + g.slack, 116 * 1024);
     { wgrad_tc_kernel<MODE><<<dim3((unsigned)g.splits, (unsigned)g.ngroups), WG_NT, smem, st>>>(tx0, tx1, tg, a, g); count_launch(); }
