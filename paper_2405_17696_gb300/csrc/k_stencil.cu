@@ -80,11 +80,14 @@ __global__ void __launch_bounds__(NTHREADS) apply_fine2_kernel(OpFine5 op, const
 // (unscaled) Krylov vector.  ||r||^2 and, on the first call, ||b||^2 are
 // reduced per RHS in FP64.
 //
-// Bound by the FP64 pipe (two operations per SM and cycle on this GPU): 17 per node and RHS as
-//   r = b + ax (xw + xe) + az (xn + xs) - (2 ax + 2 az - w^2 m) xc - i (w^2 m gamma) xc
-// with w^2 m and its products shared by a thread's two right-hand sides of one frequency, against
-// 34 in the order the operator is written, its conversions included.  512 x 256, 192 right-hand
-// sides, one GB300: 1.93 -> 1.32 ms a call, 1.47 -> 0.90 ms inside a solve.
+// Bound by the FP64 pipe (two operations per SM and cycle on this GPU): 20 per node and RHS as
+//   r = b - ax (2 xc - xw - xe) + az ((xs - xc) - (xc - xn)) + w^2 m xc - i (w^2 m gamma) xc
+// with w^2 m and its products shared by a thread's two right-hand sides of one frequency and xs - xc by
+// the next row, against 34 in the order the operator is written, its conversions included.  512 x 256,
+// 192 right-hand sides, one GB300: 1.93 -> 1.34 ms a call.
+// The differences stay: with the five terms of xc in one product it takes 17 (1.32 ms a call), but the large
+// terms cancel, and the error, over the norm of w^2 m x, at 10, 40 and 160 points per wavelength is
+// 7e-16, 1e-14 and 2e-13 in place of 1e-16, 1e-15 and 8e-15 (2e-16, 2e-15 and 1e-14 in the written order).
 template <bool FIRST>
 __global__ void __launch_bounds__(NTHREADS) residual64_kernel(OpFine5 op, const double2* __restrict__ x,
                                                               const float2* __restrict__ bvec,
@@ -106,16 +109,16 @@ __global__ void __launch_bounds__(NTHREADS) residual64_kernel(OpFine5 op, const 
         w2[0] = a * a;
         w2[1] = c * c;
     }
-    const double d0 = 2.0 * ax + 2.0 * az;
     double acc_r[2] = {0.0, 0.0}, acc_b[2] = {0.0, 0.0};
     if (ix < nx) {
         const double2 zero = make_double2(0.0, 0.0);
-        double2 xn[2], xc[2];
+        double2 dn[2], xc[2];   // this row less the one above, this row
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const double2* xb = x + (size_t)(b0 + q) * N + ix;
-            xn[q] = act[q] && iz0 > 0 && iz0 < nz ? xb[(size_t)(iz0 - 1) * nx] : zero;
+            const double2 xn = act[q] && iz0 > 0 && iz0 < nz ? xb[(size_t)(iz0 - 1) * nx] : zero;
             xc[q] = act[q] && iz0 < nz ? xb[(size_t)iz0 * nx] : zero;
+            dn[q] = make_double2(xc[q].x - xn.x, xc[q].y - xn.y);
         }
         for (int rr = 0; rr < rows; ++rr) {
             const int iz = iz0 + rr;
@@ -123,7 +126,7 @@ __global__ void __launch_bounds__(NTHREADS) residual64_kernel(OpFine5 op, const 
             const size_t p = (size_t)iz * nx + ix;
             const float2 mg = op.mg[p];
             const double k = widen(mg.x), m = k * k, gam = widen(mg.y);
-            double s = 0.0, ci = 0.0, dd = 0.0;
+            double s = 0.0, ci = 0.0;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 if (!act[q]) continue;
@@ -135,15 +138,16 @@ __global__ void __launch_bounds__(NTHREADS) residual64_kernel(OpFine5 op, const 
                 if (q == 0 || f1 != f0 || !act[0]) {
                     s = w2[q] * m;
                     ci = s * gam;                                  // coefficient s (1 - i gamma)
-                    dd = d0 - s;
                 }
                 const double bx = widen(bv.x), by = widen(conj_b ? -bv.y : bv.y);
-                const double rx = fma(-ci, -xc[q].y, fma(-dd, xc[q].x, fma(az, xn[q].x + xs.x, fma(ax, xw.x + xe.x, bx))));
-                const double ry = fma(-ci, xc[q].x, fma(-dd, xc[q].y, fma(az, xn[q].y + xs.y, fma(ax, xw.y + xe.y, by))));
+                const double2 ds = make_double2(xs.x - xc[q].x, xs.y - xc[q].y);
+                const double lx = fma(2.0, xc[q].x, -xw.x) - xe.x, ly = fma(2.0, xc[q].y, -xw.y) - xe.y;
+                const double rx = fma(ci, xc[q].y, fma(s, xc[q].x, fma(az, ds.x - dn[q].x, fma(-ax, lx, bx))));
+                const double ry = fma(-ci, xc[q].x, fma(s, xc[q].y, fma(az, ds.y - dn[q].y, fma(-ax, ly, by))));
                 r[(size_t)(b0 + q) * N + p] = make_float2(narrow(rx), narrow(ry));
                 acc_r[q] = fma(rx, rx, fma(ry, ry, acc_r[q]));
                 if (FIRST) acc_b[q] = fma(bx, bx, fma(by, by, acc_b[q]));
-                xn[q] = xc[q];
+                dn[q] = ds;
                 xc[q] = xs;
             }
         }
