@@ -91,10 +91,11 @@ coarse_gmres_kernel(OpC9 op, float2* __restrict__ V, size_t vstride, float2* __r
 #pragma unroll
         for (int i = 0; i <= KMAX; ++i) acc[i] = make_float2(0.f, 0.f);
         const float2* vj = Vb + (size_t)j * vstride;
-        // two nodes per thread (n even, vectors 16-byte aligned): 16-byte loads
+        // two nodes per thread (n even, vectors 16-byte aligned): 16-byte loads; with an odd number of columns the
+        // second may be the first of the next row
         for (int p = 2 * threadIdx.x; p < n; p += 2 * CB) {
-            const int iz = p / nx, ix = p - iz * nx;
-            float2 y0 = op.apply(vj, b, ix, iz), y1 = op.apply(vj, b, ix + 1, iz);
+            const int iz = p / nx, ix = p - iz * nx, next = ix + 1 == nx ? 1 : 0;
+            float2 y0 = op.apply(vj, b, ix, iz), y1 = op.apply(vj, b, next ? 0 : ix + 1, iz + next);
             y0.x *= sj;
             y0.y *= sj;
             y1.x *= sj;
