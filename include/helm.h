@@ -562,14 +562,22 @@ int helm_profile_flops(helm_ctx* ctx, int max, double* flops, int* count);
  * cycles as single launches; so does a solve whose capture fails.  Results are
  * the same either way.  HELM_EINVAL for a null context. */
 int helm_set_graphs(helm_ctx* ctx, int on);
+/* Whether V-cycles of the context with two pre- and two post-sweeps run each leg of a level in
+ * one pass (on by default) or by a kernel per sweep and transfer, with the same results bit
+ * for bit: for comparison and diagnosis.  HELM_EINVAL for a null context. */
+int helm_set_legs(helm_ctx* ctx, int on);
 
 /* Autotuning of the multigrid sweeps' thread-block shapes (and, for a context with a
  * network, of the convolutions' tiling, cnn_autotune): runs one V-cycle on a synthetic batch
- * of nrhs right-hand sides (1 <= nrhs <= max_rhs).  The first Jacobi sweep on each grid times
- * the candidate block shapes (32x8, 64x4, 32x4, 128x2, 32x16, 16x16) with CUDA events and
- * records the fastest in a process-wide table that every later sweep on that grid uses, at
- * any batch size and in any context.  *n_shapes (may be NULL) receives the number of tuned
- * (sweep, grid) entries.  helm_setup runs it with max_rhs when opts.autotune is set. */
+ * of nrhs right-hand sides (1 <= nrhs <= max_rhs) with a kernel per sweep.  The first Jacobi
+ * sweep on each grid times the candidate block shapes (32x8, 64x4, 32x4, 128x2, 32x16, 16x16)
+ * with CUDA events and records the fastest in a process-wide table that every later such sweep
+ * on that grid uses, at any batch size and in any context: cycles with other counts than two
+ * and two sweeps, the fine sweeps of a cycle with an initial guess, a coarsest level by Jacobi
+ * sweeps, and any cycle after helm_set_legs(ctx, 0).  The cycle with two and two sweeps
+ * from zero, the default, runs each leg of a level in one pass, which has no shape to tune.
+ * *n_shapes (may be NULL) receives the number of tuned (sweep, grid) entries.  helm_setup runs
+ * it with max_rhs when opts.autotune is set. */
 int helm_autotune(helm_ctx* ctx, int nrhs, int* n_shapes);
 /* Forget every tuned block shape of the sweeps. */
 void helm_autotune_reset(void);

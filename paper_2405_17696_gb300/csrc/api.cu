@@ -269,7 +269,7 @@ int smooth_and_recurse(helm_ctx* c, const Op& op, int l, float2* u_out, const fl
     Level& L = c->lev[l];
     Level& C = c->lev[l + 1];
     const int pre = c->opt.pre, post = c->opt.post, n = pre + post;
-    if (pre == 2 && post == 2 && !u0 && !stencil_tuning_on()) {
+    if (pre == 2 && post == 2 && !u0 && c->legs && !stencil_tuning_on()) {
         // the default cycle: one pass per leg (other sweep counts and initial guesses take the kernels below,
         // whose block shapes helm_autotune times)
         HELM_TRY(launch_leg_down(c, op, f, L.t, C.f, nb, mask));
@@ -850,6 +850,12 @@ int helm_solve(helm_ctx* c, const helm_c64* rhs, helm_c128* x, int nrhs, const i
     if (result == HELM_ENOCONV) set_error("some right-hand sides did not reach tol within max_iter");
     if (result == HELM_EBREAKDOWN) set_error("breakdown (NaN/Inf) in some right-hand sides");
     return result;
+}
+
+int helm_set_legs(helm_ctx* c, int on) {
+    if (!c) { set_error("helm_set_legs: null context"); return HELM_EINVAL; }
+    c->legs = on != 0;
+    return HELM_OK;
 }
 
 int helm_set_graphs(helm_ctx* c, int on) {

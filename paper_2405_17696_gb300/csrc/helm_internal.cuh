@@ -266,6 +266,7 @@ struct helm_ctx {
     // restart cycles of MG-preconditioned (or plain) FGMRES are captured once per solve
     // as a CUDA graph on capture_stream and replayed on stream (helm_set_graphs)
     int graphs = 1;
+    int legs = 1;   // the 2 + 2 sweep cycle in one pass per leg (helm_set_legs)
     cudaStream_t capture_stream = nullptr;
     std::vector<float> omega;       // host copy (rad/s)
     float2* mg = nullptr;           // [nz][nx] {kappa, gamma}
@@ -395,7 +396,7 @@ void cnn_ctx_free(helm_ctx* c);
 int cnn_ctx_precondition(helm_ctx* c, float2* z, const float2* v, int nb, const int* mask, int with_vcycle);
 int cnn_ctx_compact(helm_ctx* c, int nb);   // list the RHS still running (flags in cnn_act_host)
 void cnn_retrain_free(helm_ctx* c);         // cnn_retrain.cu
-// Block-shape autotuning of the Jacobi sweeps (k_multigrid.cu): while on, the first launch
+// Block-shape autotuning of the separate Jacobi sweeps (k_multigrid.cu): while on, the first launch
 // on a grid times the candidate shapes and records the fastest (process-wide table).
 void stencil_tuning(bool on);
 bool stencil_tuning_on();

@@ -140,6 +140,8 @@ def _load():
     lib.cnn_autotune_reset.restype = None
     lib.helm_set_graphs.argtypes = [vp, ip]
     lib.helm_set_graphs.restype = ip
+    lib.helm_set_legs.argtypes = [vp, ip]
+    lib.helm_set_legs.restype = ip
     lib.cnn_set_conv_ring.argtypes = [ip, ip]
     lib.cnn_set_conv_ring.restype = ip
     lib.cnn_conv_narrow_launches.argtypes = []
@@ -487,6 +489,11 @@ def helm_launch_count() -> int:
 def helm_set_graphs(ctx, on: bool):
     """Capture and replay the restart cycles of MG / plain FGMRES as a CUDA graph (default on)."""
     _check(lib.helm_set_graphs(ctx, 1 if on else 0), "helm_set_graphs")
+
+
+def helm_set_legs(ctx, on: bool):
+    """V-cycles with 2 + 2 sweeps in one pass per leg (default) or a kernel per sweep: the same bits."""
+    _check(lib.helm_set_legs(ctx, 1 if on else 0), "helm_set_legs")
 
 
 # --------------------------------------------------------------------------
