@@ -79,6 +79,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "helm_internal.cuh"
@@ -812,8 +813,10 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
                 tile_coords(k, b, xs, ys);
                 const uint32_t dbase = lane_base + (uint32_t)acc * g.acc_cols;
                 const size_t img_base = (size_t)b * (size_t)(a.npad >> 3) * (size_t)hw_out * 8;
-                // output pixel of this thread's row of block bi (-1: none)
-                auto pixel = [&](int bi) {
+                // output pixel of this thread's row of block bi (-1: none); an up-sampled image may have more than 2^31
+                // (see plan_launch)
+                using Pixel = std::conditional_t<MODE == 2 || MODE == 3, long long, int>;
+                auto pixel = [&](int bi) -> Pixel {
                     if (bi >= nblk) return -1;
                     const int ph = MODE == 5 ? 0 : bi / g.mb, m = bi - ph * g.mb;
                     int yy = m, xx = row;        // mode 5: a block is an output row
@@ -827,22 +830,22 @@ __global__ void __launch_bounds__(threads_of(MODE), 2) conv3x3_tma_kernel(const 
                         oy = 2 * oy + (g.psplit ? tile_py(k) : ph >> 1);
                         ox = 2 * ox + (g.psplit ? ph : ph & 1);
                     }
-                    return xx < g.tw && yy < g.rows && oy < a.hout && ox < a.wout ? oy * a.wout + ox : -1;
+                    return xx < g.tw && yy < g.rows && oy < a.hout && ox < a.wout ? (Pixel)oy * a.wout + ox : (Pixel)-1;
                 };
                 // (16 channels: the next block's operand is under way while this one is finished)
-                int pix = pixel(wg);
+                Pixel pix = pixel(wg);
                 Pre2 pre{};
-                if (ACT && a.npad == 16) pre = preload(img_base + (size_t)(unsigned)pix * 8, 0, pix >= 0);
+                if (ACT && a.npad == 16) pre = preload(img_base + (size_t)pix * 8, 0, pix >= 0);
                 if (!wait_bar(&tfull[acc], par, abort_v, 128)) { *abort_v = 1; break; }
                 tc::tc_fence_after_sync();
                 for (int bi = wg; bi < nblk; bi += 2) {
-                    const int next = pixel(bi + 2);
-                    const size_t ob = img_base + (size_t)(unsigned)pix * 8;   // channel 0 of this pixel
+                    const Pixel next = pixel(bi + 2);
+                    const size_t ob = img_base + (size_t)pix * 8;   // channel 0 of this pixel
                     const long long p = (long long)b * hw_out + pix;
                     const uint32_t tcol = dbase + (uint32_t)((MODE == 5 ? g.rows - 1 - bi : bi) * a.npad);
                     if (a.npad == 16) {
                         Pre2 pn{};
-                        if (ACT) pn = preload(img_base + (size_t)(unsigned)next * 8, 0, next >= 0);
+                        if (ACT) pn = preload(img_base + (size_t)next * 8, 0, next >= 0);
                         else pre = preload(ob, 0, pix >= 0);
                         float v[16];
                         tc::tmem_ld16(tcol, v);
