@@ -121,11 +121,12 @@ __global__ void transpose_weights_kernel(const __nv_bfloat16* __restrict__ W, in
 // The 2x2 sums of fine [nb][2h][2w][c] (c a multiple of 8) as an input gradient (see GradOut): a thread per
 // coarse pixel and 8-channel chunk, the chunks of a pixel side by side (a warp reads whole runs of `fine`;
 // with a chunk per block each run was fetched in 32-byte pieces: 1024 x 512, 32 channels, 16 images, one GB300:
-// 569 -> 232 us), 16-byte accesses; grid (pixels x chunks, images).
-__global__ void sumpool_grad_kernel(const float* __restrict__ fine, int h, int w, int c, GradOut o) {
-    const long long b = blockIdx.y, hw = (long long)h * w;
+// 569 -> 232 us), 16-byte accesses; grid (pixels x chunks, images), each in strides.
+__global__ void sumpool_grad_kernel(const float* __restrict__ fine, int nb, int h, int w, int c, GradOut o) {
+    const long long hw = (long long)h * w;
     const size_t row = 2 * (size_t)w * c;                     // a fine row
     const unsigned nc8s = (unsigned)c >> 3;
+    for (long long b = blockIdx.y; b < nb; b += gridDim.y)
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < hw * nc8s;
          i += (long long)gridDim.x * blockDim.x) {
         const long long pix = i / nc8s;
@@ -494,7 +495,7 @@ int layer_dgrad(const __nv_bfloat16* g, int npad, const __nv_bfloat16* W, int ci
     LaunchScope scope(prof_ctx, K_CNN_IO);
     const long long hw = (long long)hin * win;
     const unsigned gx = (unsigned)std::max<long long>(1, std::min<long long>((hw * (cp / 8) + 255) / 256, std::max(1, 9728 / nb)));
-    { sumpool_grad_kernel<<<dim3(gx, (unsigned)nb), 256, 0, st>>>(fine, hin, win, cp, out); count_launch(); }
+    { sumpool_grad_kernel<<<dim3(gx, (unsigned)std::min(nb, 65535)), 256, 0, st>>>(fine, nb, hin, win, cp, out); count_launch(); }
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_ECUDA;
 }
 
@@ -612,7 +613,7 @@ class Backward {
                 if (cg == L.npad && cg % 8 == 0)
                     { mask_to_bf16_vec_kernel<<<dim3((unsigned)bx, (unsigned)(cg / 8), (unsigned)op.nb), 256, 0, st_>>>(
                         Gy, ymask, L.npad, L.npad, hw, gw, rg, had); count_launch(); }
-                else if (cg <= 8 && L.npad == 16 && !ymask && !rg)
+                else if (cg <= 8 && L.npad == 16 && !ymask && !rg && op.nb <= 65535)
                     { narrow_to_bf16_kernel<<<dim3((unsigned)bx, (unsigned)op.nb), 256, 0, st_>>>(Gy, cg, hw, gw); count_launch(); }
                 else
                     { mask_to_bf16_kernel<<<1184, 256, 0, st_>>>(Gy, cg, ymask, L.npad, L.npad, nout, hw, gw, rg, had); count_launch(); }
