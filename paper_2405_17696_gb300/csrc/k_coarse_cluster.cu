@@ -597,10 +597,11 @@ int launch_coarse_cluster(const helm_ctx* c, int level, const float2* f, float2*
     const int k = c->opt.coarse_iters;
     const CoarsePlan p = coarse_plan_cached(L.nx, L.nz, k, nb);
     if (!p.npt) return HELM_EUNSUPPORTED;
-    const unsigned long long kk = (unsigned long long)k;
     LaunchScope scope(c, K_COARSE_GMRES);
-    // as the other coarsest solve counts: ||f||, per step 2 (j + 1) basis reads, v_j, w, v_{j+1}, the combination
-    const Tally tl = tally(c, K_COARSE_GMRES, 8ull * Nc * (kk * kk + 5 * kk + 2));
+    // f in, u out; of n spilled vectors each is written once and read twice in its own step and every later one, and
+    // once for the combination: n^2 + 3 n
+    const unsigned long long n = (unsigned long long)(k - p.nsm);
+    const Tally tl = tally(c, K_COARSE_GMRES, 8ull * Nc * (2 + n * n + 3 * n));
     const OpC9 op = coarse_op(c, level);
     const size_t vs = (size_t)c->cap * Nc;
     switch (p.npt) {
