@@ -11,16 +11,18 @@
 //
 // A warp marches down a strip of 64 columns of one right-hand side.  A lane holds a pair
 // of columns (2k, 2k + 1); its neighbours' values come by shuffles, and the last three rows
-// of every intermediate field stay in registers, so there is no shared memory and no
-// barrier.  The strip's outer columns and the first and last rows of a segment are
+// of every intermediate field stay in registers: shared memory holds only the rows that are
+// read, copied ahead.  The strip's outer columns and the first and last rows of a segment are
 // computed twice, by the neighbours too: 29 (down) or 30 (up) of 32 lanes and all but 5 or
 // 4 rows of a segment are written.  Values outside the grid are set to zero.  Every node is
-// computed by the same operations in the same order as by the separate kernels.  The warps of a block take different right-hand sides of the same
-// tile.  On a coarse level they share the nine coefficients of its nodes in shared memory
-// (read per warp they are four times the traffic of the fields); right-hand sides of
-// different frequencies in a block take turns.  On the fine grid the medium is an eighth
-// of that and a barrier per row costs more than it saves (139 -> 162 us at 512 x 256, 192
-// right-hand sides), so every warp reads its own.
+// computed by the same operations in the same order as by the separate kernels.
+//
+// The warps of a block take different right-hand sides of the same tile.  On a coarse level
+// they share the nine coefficients of its nodes (read per warp they are four times the
+// traffic of the fields), at a barrier per row; right-hand sides of different frequencies in
+// a block take turns.  On the fine grid the medium is an eighth of that and such a barrier
+// costs more than it saves (139 -> 162 us at 512 x 256, 192 right-hand sides), so every warp
+// reads its own and only the warp waits for its copies.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
